@@ -275,7 +275,8 @@ int malt_set_ns_schedule(malt_state_t* st, int32_t schedule);
 
 /* Host only (no GPU, no CUDA call): the work table of the persistent schedule
  * for these parameter shapes (only rows and cols are read) and ns_steps
- * iterations, in claim order, 8 int32 per item: launch group, stage (3 i +
+ * iterations with every matrix in the iterated form (malt_ns_plan says which
+ * form a matrix takes), in claim order, 8 int32 per item: launch group, stage (3 i +
  * kind for iteration i), kind (0 Gram, 1 Poly, 2 B*X), matrix index, local
  * index (the 256 x 256 tile of the NS frame; Gram and Poly list the upper
  * triangle only), the index of the counter the item waits for
@@ -287,6 +288,27 @@ int malt_set_ns_schedule(malt_state_t* st, int32_t schedule);
  * MALT_ERR_UNSUPPORTED for a shape malt_init_state would reject. */
 int malt_ns_schedule(const malt_param_t* params, int32_t n, int32_t ns_steps, int32_t* out,
                      int64_t capacity, int64_t* count);
+
+/* Host only: the products that a step runs on each matrix of a set of n
+ * rows x cols matrices, in order.
+ * An operation is out = gamma k^kx (a b) + beta e + alpha I with
+ * k = 1 / (||Mt||_F + ns_eps), buffers numbered 0 .. 3 (p x p), 4 and 5 (the
+ * iterates X; 4 holds Mt on the wide orientation, in bf16, at the start) and 6
+ * (O), -1 for none; its operands are fp16 or bf16, its output is rounded to
+ * fp16 or bf16.  kind 0 is a X X^T, 1 a product of two symmetric p x p
+ * matrices (both kinds computed as an upper triangle and mirrored), 2 a product
+ * of a p x p matrix with X.  Writes min(capacity, total) operations and the
+ * total to *count.  MALT_ERR_INVALID_ARG for bad arguments,
+ * MALT_ERR_UNSUPPORTED for a shape malt_init_state would reject. */
+typedef struct {
+    int32_t kind;
+    int32_t in_f16, out_f16;
+    int32_t a, b, e, out;
+    int32_t kx;
+    float alpha, beta, gamma;
+} malt_ns_op_t;
+int malt_ns_plan(int64_t rows, int64_t cols, int32_t n, const malt_hparams_t* hp, malt_ns_op_t* out,
+                 int32_t capacity, int32_t* count);
 
 /* Statistics stage of ONE matrix without any device allocation.
  * The paper has no counterpart: this exists for callers that cannot allocate

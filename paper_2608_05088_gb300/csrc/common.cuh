@@ -95,10 +95,49 @@ enum NsMode : int32_t { kNsPhased = 0, kNsPersistent = 1 };
 // Epilogue warps of a CTA pair; each one signals a finished item once.
 constexpr uint32_t kNsSignalsPerTile = 2 * kEpiWarpsPerCta;
 
-// Stages of a persistent work table: the products of Newton-Schulz
-// iteration i are stages 3 i + {kGram, kPoly, kBX}.  The table of k
-// iterations is the first k iterations' entries of any longer table.
+// Stages of a persistent work table: operation s of a matrix's form.  In the
+// iterated form the products of iteration i are stages 3 i + {kGram, kPoly,
+// kBX}, and the table of k iterations is the first k iterations' entries of any
+// longer one.
 constexpr int kMaxNsSteps = 64;
+
+// Buffers of a class that an operation reads or writes: the p x p matrices
+// 0 .. 3 (0 holds A, 1 holds B' in the iterated form), the two iterates X, and
+// the last iterate O.
+constexpr int8_t kBufX = 4, kBufO = 6, kBufNone = -1;
+
+// One product of a Newton-Schulz run:
+//   out = gamma k^kx (a b) + beta e + alpha I
+// with a read as K-major rows, b as K-major rows (Gram and p x p products; the
+// p x p matrices are symmetric) or MN-major (kBX), and k = 1 / (||Mt|| + ns_eps).
+struct NsOp {
+    int8_t kind;            // GemmPhase: kGram X X^T (K = q), kPoly a p x p product (K = p), kBX
+    int8_t f16, out16;      // operands (and e) fp16 instead of bf16; the output
+    int8_t a, b, e, out;    // buffers
+    int8_t kx;              // power of k that scales the product
+    float alpha, beta, gamma;
+};
+
+// Operations of the longest grouped run (8 iterations in groups 1, 2, 2, 3).
+constexpr int kMaxGroupedOps = 32;
+
+// Product `kind` of iteration `iter` of the iterated form (X <- B' X).
+__host__ __device__ __forceinline__ NsOp ns_iterated_op(int32_t iter, int32_t kind, bool last, float a,
+                                                        float b, float c) {
+    const int8_t cur = static_cast<int8_t>(kBufX + (iter & 1));
+    NsOp o;
+    o.kind = static_cast<int8_t>(kind);
+    o.f16 = o.out16 = 0;
+    o.kx = iter > 0 ? 0 : kind == kGram ? 2 : kind == kBX ? 1 : 0;
+    o.a = kind == kGram ? cur : kind == kPoly ? 0 : 1;
+    o.b = kind == kPoly ? 0 : cur;
+    o.e = kind == kPoly ? 0 : kBufNone;
+    o.out = kind == kGram ? 0 : kind == kPoly ? 1 : last ? kBufO : static_cast<int8_t>(kBufX + ((iter & 1) ^ 1));
+    o.alpha = kind == kPoly ? a : 0.f;
+    o.beta = kind == kPoly ? b : 0.f;
+    o.gamma = kind == kPoly ? c : 1.f;
+    return o;
+}
 
 // One item of a persistent work table.
 struct __align__(16) NsEntry {
@@ -115,35 +154,38 @@ __host__ __device__ __forceinline__ int32_t entry_b(const NsEntry& e) {
 }
 
 // One shape class (every matrix whose NS frame is p x q, stored batched) with
-// all the tensor maps of the three products of an NS iteration.
+// the tensor maps of all its buffers.
 struct NsClass {  // 64-byte aligned through its CUtensorMap members
-    CUtensorMap tmX[2];           // the ping-pong iterates X as K-major rows (box kBK x kBM)
-    CUtensorMap tmXmn[2];         // the same buffers as an MN-major [K][N] operand (box kBMN x kBK)
-    CUtensorMap tmA, tmB;         // A = X X^T and B' = aI + bA + cA^2, K-major rows
-    CUtensorMap stX[2], stA, stB, stO;   // epilogue stores: box 32 x 32, 64-byte swizzle
+    CUtensorMap tmK[6];           // p x p buffers 0 .. 3 and the iterates X as K-major rows (box kBK x kBM)
+    CUtensorMap tmXmn[2];         // the iterates as an MN-major [K][N] operand (box kBMN x kBK)
+    CUtensorMap stK[6], stO;      // epilogue stores of the same buffers and of O: box 32 x 32, 64-byte swizzle
     CUtensorMap stOt;             // the O buffer as [q][p]: a tall W's O, stored in W's layout
     int32_t p, q, batch;
     int32_t tiles_p, tiles_q;     // 256-wide tiles along p and along q
-    int32_t sym_begin;            // first item of this class within a Gram or Poly phase
-    int32_t full_begin;           // first item of this class within a BX phase
+    int32_t item_begin;           // first item of this class in a phased launch
+    int32_t can_group;            // the shape takes the grouped form when the run may
+    int32_t grouped;              // this run's form
     int32_t bx_col_major;         // list B*X tiles column by column (X larger than kBxColBytes)
     const int32_t* mat_of;        // [batch] -> matrix index
-    const __nv_bfloat16* A;       // the A buffer [batch][p][p] (read by the Poly epilogue)
+    const uint16_t* A;            // p x p buffer 0 [batch][p][p], 16-bit (read by the H epilogue)
 };
 
-// Work list of one launch: for each NS iteration i, the Gram tiles of every
-// class (sym_items), then the Poly tiles (sym_items), then the BX tiles
-// (full_items); item s-phase index = 3 i + kind.  A launch runs the items
-// [item_begin, item_end): one phase (phased schedule, static round-robin) or
-// the whole list (persistent schedule, claimed through *queue, each tile
-// waiting for its matrix's previous phase in done[]).
+// Work list of one launch.  Each class runs its form's operations in order
+// (stage s = operation s); within a stage the items are the tiles of every
+// class, batch slot by batch slot.  A phased launch runs one stage (items
+// [0, item_end), static round-robin, class c's from cls[c].item_begin); a
+// persistent launch runs all of them from a work table (claimed through
+// *queue, each tile waiting for its matrix's previous stage in done[]).
 struct NsParams {
     NsClass cls[kMaxClasses];
+    NsOp ops[kMaxGroupedOps];     // the grouped form's operations
+    int32_t nops;                 // their number (0: no class runs grouped)
     int32_t nclasses;
     int32_t nmat;                 // size of one row of done[]
     int32_t ns_steps;
-    int32_t sym_items, full_items;
-    int32_t item_begin, item_end;
+    int32_t stage;                // phased launch: the stage it runs
+    int32_t item_end;             // items of the launch
+    int32_t sym_items, full_items;   // tiles of a symmetric product, of B*X, over all classes
     float a, b, c;
     const MatDesc* mats;
     MatScalars* scal;
@@ -151,16 +193,23 @@ struct NsParams {
     uint32_t* queue;              // next unclaimed item (persistent schedule)
     uint32_t* done;               // [stages][nmat] finished-item signals (persistent)
     uint64_t budget_ns;
-    // Persistent launches: the work table (item_end entries) and its stages.
-    const NsEntry* table;
-    int32_t nstages;              // 3 ns_steps
+    const NsEntry* table;         // persistent launches: the work table (item_end entries)
 };
 static_assert(sizeof(NsParams) <= 32764, "NsParams is passed by value as the kernel parameter");
 
+// Number of operations of a class in this launch's run, and operation s.
+__host__ __device__ __forceinline__ int32_t ns_num_stages(const NsParams& P, const NsClass& C) {
+    return C.grouped ? P.nops : 3 * P.ns_steps;
+}
+__host__ __device__ __forceinline__ NsOp ns_op(const NsParams& P, const NsClass& C, int32_t s) {
+    if (C.grouped) return P.ops[s];
+    const int32_t iter = s / 3;
+    return ns_iterated_op(iter, s - 3 * iter, iter == P.ns_steps - 1, P.a, P.b, P.c);
+}
+
 // One decoded work item: a 256 x 256 output tile of one product.
 struct NsWork {
-    int32_t s;                    // 3 * iter + kind
-    int32_t iter, kind;
+    NsOp op;
     int32_t cls, b;               // class and batch slot (matrix = cls.mat_of[b])
     int32_t mt, nt;               // tile row / column
     int32_t local;                // tile index within the matrix's product
@@ -210,32 +259,20 @@ __host__ __device__ __forceinline__ int32_t mat_apply_blocks(const MatDesc& d) {
     return static_cast<int32_t>((static_cast<int64_t>(d.m) * d.n + kApplyElems - 1) / kApplyElems);
 }
 
+// Item `item` of a phased launch (stage P.stage of every class that has it).
 __host__ __device__ __forceinline__ NsWork ns_decode(const NsParams& P, int32_t item) {
     NsWork w;
-    const int32_t per_iter = 2 * P.sym_items + P.full_items;
-    w.iter = item / per_iter;
-    int32_t r = item - w.iter * per_iter;
-    if (r < P.sym_items) {
-        w.kind = kGram;
-    } else if (r < 2 * P.sym_items) {
-        w.kind = kPoly;
-        r -= P.sym_items;
-    } else {
-        w.kind = kBX;
-        r -= 2 * P.sym_items;
-    }
-    w.s = 3 * w.iter + w.kind;
-    const bool sym = w.kind != kBX;
     int32_t c = 0;
-    while (c + 1 < P.nclasses && r >= (sym ? P.cls[c + 1].sym_begin : P.cls[c + 1].full_begin)) ++c;
+    while (c + 1 < P.nclasses && item >= P.cls[c + 1].item_begin) ++c;
     const NsClass& C = P.cls[c];
-    const int32_t local = r - (sym ? C.sym_begin : C.full_begin);
-    const int32_t per = ns_phase_tiles(C, w.kind);
+    w.op = ns_op(P, C, P.stage);
+    const int32_t local = item - C.item_begin;
+    const int32_t per = ns_phase_tiles(C, w.op.kind);
     w.cls = c;
     w.b = local / per;
     const int32_t rem = local - w.b * per;
     w.local = rem;
-    ns_tile_coords(C, w.kind, rem, &w.mt, &w.nt);
+    ns_tile_coords(C, w.op.kind, rem, &w.mt, &w.nt);
     return w;
 }
 

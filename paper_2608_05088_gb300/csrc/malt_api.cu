@@ -28,6 +28,7 @@
 #include "../../include/malt.h"
 #include "common.cuh"
 #include "kernels.h"
+#include "ns_plan.h"
 
 using namespace malt;
 
@@ -80,13 +81,15 @@ struct ShapeClass {
     int p = 0, q = 0, batch = 0;
     std::vector<int> mats;
     int32_t* d_mat_of = nullptr;
+    bool can_group = false;                      // ns_grouped_shape
     __nv_bfloat16* X[2] = {nullptr, nullptr};   // ping-pong NS iterates [batch][p][q]
-    __nv_bfloat16* A = nullptr;                  // X X^T        [batch][p][p]
-    __nv_bfloat16* B = nullptr;                  // aI + bA + cA^2 [batch][p][p]
+    // p x p matrices [batch][p][p]: A, B' (or H), and for classes that can
+    // take the grouped form two more (H A and the running product)
+    __nv_bfloat16* P[4] = {nullptr, nullptr, nullptr, nullptr};
     __nv_bfloat16* O = nullptr;                  // last iterate, per matrix in W's layout:
                                                  // [p][q] (wide) or [q][p] (tall)
-    CUtensorMap tmX[2], tmXmn[2], tmA, tmB;    // 128-row K-major boxes; 64x64 MN boxes
-    CUtensorMap stX[2], stA, stB, stO, stOt;   // epilogue store maps (stOt: O as [q][p])
+    CUtensorMap tmK[6] = {}, tmXmn[2];          // 128-row K-major boxes; 64x64 MN boxes
+    CUtensorMap stK[6] = {}, stO, stOt;         // epilogue store maps (stOt: O as [q][p])
 };
 
 // Workspace carving: 256-byte aligned buffers, each followed by a guard
@@ -166,11 +169,17 @@ struct malt_state {
     uint32_t* d_sched = nullptr;
     int sched_groups_pad = 0;
     int ns_schedule = MALT_NS_AUTO;
-    // Work table of the persistent launches, one per launch group, for
-    // kMaxNsSteps iterations (in the workspace, uploaded at init); a launch of
-    // k iterations claims its first k * table_per_iter[group] entries.
-    std::vector<NsEntry*> table_dev;
-    std::vector<int32_t> table_per_iter;
+    // Work tables of the persistent launches, per launch group (in the
+    // workspace, uploaded at init).  Iterated form: one for kMaxNsSteps
+    // iterations, of which a run of k claims the first k * per_iter entries.
+    // Grouped form: one per k.
+    struct NsTables {
+        NsEntry* iterated = nullptr;
+        int32_t per_iter = 0;
+        NsEntry* grouped[kMaxGroupedSteps + 1] = {};
+        int32_t grouped_items[kMaxGroupedSteps + 1] = {};
+    };
+    std::vector<NsTables> tables;
     int32_t last_timeout[5] = {};   // site record of the last timeout malt_check reported
     uint64_t* d_guard_off = nullptr;   // byte offsets of the guard regions
     unsigned long long* d_guard_bad = nullptr;   // corrupted guard bytes found by the check
@@ -295,6 +304,7 @@ struct LaunchScope {
 };
 
 constexpr int kMaxStages = 3 * kMaxNsSteps;
+static_assert(kMaxStages >= kMaxGroupedOps, "one row of counters per stage");
 // Auto schedule: persistent when a symmetric product has fewer tiles than
 // this many waves of the resident CTA pairs.
 constexpr int kAutoPersistentWaves = 16;
@@ -340,6 +350,12 @@ void build_classes(const malt_param_t* params, int n, std::vector<MatDesc>& hmat
         d.pre_tc = (c + kPreCols - 1) / kPreCols;
         d.ns_tiles = ((p + kTileM - 1) / kTileM) * ((q + kBN - 1) / kBN);
     }
+    int64_t tiles = 0;                 // of one symmetric product over the set
+    for (const ShapeClass& C : classes) {
+        const int64_t tp = (C.p + kTileM - 1) / kTileM;
+        tiles += tp * (tp + 1) / 2 * C.batch;
+    }
+    for (ShapeClass& C : classes) C.can_group = ns_grouped_shape(C.p, C.q, tiles);
 }
 
 // Newton-Schulz work lists: classes ordered by Gram reduction length (q, then
@@ -368,15 +384,12 @@ void plan_ns_groups(const std::vector<ShapeClass>& classes, int nmat, std::vecto
             const ShapeClass& S = classes[order[start + j]];
             if (slot_class != nullptr) slot_class->back().push_back(order[start + j]);
             NsClass& C = P.cls[j];
-            for (int b = 0; b < 2; ++b) {
-                C.tmX[b] = S.tmX[b];
-                C.tmXmn[b] = S.tmXmn[b];
-                C.stX[b] = S.stX[b];
+            for (int b = 0; b < 6; ++b) {
+                C.tmK[b] = S.tmK[b];
+                C.stK[b] = S.stK[b];
             }
-            C.tmA = S.tmA;
-            C.tmB = S.tmB;
-            C.stA = S.stA;
-            C.stB = S.stB;
+            for (int b = 0; b < 2; ++b) C.tmXmn[b] = S.tmXmn[b];
+            C.can_group = S.can_group ? 1 : 0;
             C.stO = S.stO;
             C.stOt = S.stOt;
             C.p = S.p;
@@ -384,11 +397,9 @@ void plan_ns_groups(const std::vector<ShapeClass>& classes, int nmat, std::vecto
             C.batch = S.batch;
             C.tiles_p = (S.p + kTileM - 1) / kTileM;
             C.tiles_q = (S.q + kBN - 1) / kBN;
-            C.sym_begin = sym;
-            C.full_begin = full;
             C.bx_col_major = static_cast<int64_t>(S.p) * S.q * 2 > kBxColBytes ? 1 : 0;
             C.mat_of = S.d_mat_of;
-            C.A = S.A;
+            C.A = reinterpret_cast<const uint16_t*>(S.P[0]);
             sym += ns_phase_tiles(C, kGram) * S.batch;
             full += ns_phase_tiles(C, kBX) * S.batch;
         }
@@ -403,21 +414,26 @@ void plan_ns_groups(const std::vector<ShapeClass>& classes, int nmat, std::vecto
 // Tiles of one matrix in one product of this kind.
 int32_t stage_items(int kind, const NsClass& C) { return ns_phase_tiles(C, kind); }
 
-// The work table of one launch group for k iterations: for each product of
-// each iteration, every tile of every class (slot order), batch slot by
-// batch slot.  Every item depends on the previous product of its own matrix,
-// listed earlier: claiming in table order never waits on an item that has
-// not been claimed.  The table of k iterations is the prefix of any longer
-// one (an iteration adds entries at the end and changes none before it).
+// The work table of one launch group for a run of k iterations: for each
+// stage, every tile of every class that has the stage (slot order), batch slot
+// by batch slot.  Every item depends on the previous stage of its own matrix,
+// listed earlier: claiming in table order never waits on an item that has not
+// been claimed.  With every class in the iterated form the table of k
+// iterations is the prefix of any longer one (an iteration adds entries at the
+// end and changes none before it); G.cls[].grouped picks the form and G.ops
+// holds the grouped one's operations.
 void build_table(const NsParams& G, const std::vector<int>& slot_class,
-                 const std::vector<ShapeClass>& classes, int k, std::vector<NsEntry>& out) {
+                 const std::vector<ShapeClass>& classes, std::vector<NsEntry>& out) {
     out.clear();
-    for (int st = 0; st < 3 * k; ++st) {
-        const int kind = st % 3;
+    int stages = 0;
+    for (int c = 0; c < G.nclasses; ++c) stages = std::max(stages, ns_num_stages(G, G.cls[c]));
+    for (int st = 0; st < stages; ++st) {
         for (int c = 0; c < G.nclasses; ++c) {
+            const NsClass& C = G.cls[c];
+            if (st >= ns_num_stages(G, C)) continue;
             const ShapeClass& S = classes[slot_class[c]];
-            const int32_t items = stage_items(kind, G.cls[c]);
-            const int32_t prev = st == 0 ? 0 : stage_items((st - 1) % 3, G.cls[c]);
+            const int32_t items = stage_items(ns_op(G, C, st).kind, C);
+            const int32_t prev = st == 0 ? 0 : stage_items(ns_op(G, C, st - 1).kind, C);
             for (int b = 0; b < S.batch; ++b) {
                 for (int t = 0; t < items; ++t) {
                     NsEntry e;
@@ -432,7 +448,24 @@ void build_table(const NsParams& G, const std::vector<int>& slot_class,
     }
 }
 
-// Entries per iteration of a launch group's table.
+// Set a launch group up for a run of k iterations with these coefficients:
+// the classes that can take the grouped form do, when the run may.
+void set_run(NsParams& G, int k, float a, float b, float c, bool grouped) {
+    G.ns_steps = k;
+    G.a = a;
+    G.b = b;
+    G.c = c;
+    G.nops = grouped ? ns_grouped_ops(k, a, b, c, G.ops) : 0;
+    for (int j = 0; j < G.nclasses; ++j) G.cls[j].grouped = grouped ? G.cls[j].can_group : 0;
+}
+
+bool any_grouped(const NsParams& G) {
+    for (int c = 0; c < G.nclasses; ++c)
+        if (G.cls[c].can_group) return true;
+    return false;
+}
+
+// Entries per iteration of a launch group's iterated-form table.
 int32_t table_per_iter(const NsParams& G) { return 2 * G.sym_items + G.full_items; }
 
 int plan_and_allocate(malt_state* st, const malt_param_t* params, int n) {
@@ -454,15 +487,16 @@ int plan_and_allocate(malt_state* st, const malt_param_t* params, int n) {
         o_ns[i] = cv.take(sizeof(float) * 2 * kNsPartsPerTile * static_cast<size_t>(d.ns_tiles));
     }
     const int nc = static_cast<int>(st->classes.size());
-    std::vector<size_t> o_X0(nc), o_X1(nc), o_A(nc), o_B(nc), o_O(nc), o_matof(nc);
+    std::vector<size_t> o_X0(nc), o_X1(nc), o_O(nc), o_matof(nc);
+    std::vector<size_t> o_P[4];
+    for (auto& o : o_P) o.resize(nc);
     for (int k = 0; k < nc; ++k) {
         const ShapeClass& C = st->classes[k];
         const size_t pq = static_cast<size_t>(C.batch) * C.p * C.q * 2;
         const size_t pp = static_cast<size_t>(C.batch) * C.p * C.p * 2;
         o_X0[k] = cv.take(pq);
         o_X1[k] = cv.take(pq);
-        o_A[k] = cv.take(pp);
-        o_B[k] = cv.take(pp);
+        for (int j = 0; j < (C.can_group ? 4 : 2); ++j) o_P[j][k] = cv.take(pp);
         o_O[k] = cv.take(pq);
         o_matof[k] = cv.take(sizeof(int32_t) * C.batch);
     }
@@ -481,15 +515,27 @@ int plan_and_allocate(malt_state* st, const malt_param_t* params, int n) {
                                                        static_cast<size_t>(kMaxStages) * n));
     // Persistent work tables for kMaxNsSteps iterations, one per launch group
     // (planned here without tensor maps, which only the launches need).
+    // The grouped form's tables depend on k, so a group with a class that can
+    // take it gets one for each k it covers.
     std::vector<std::vector<NsEntry>> tables;
     {
         std::vector<NsParams> groups;
         std::vector<std::vector<int>> slot_class;
         plan_ns_groups(st->classes, n, groups, &slot_class);
-        tables.resize(groups.size());
         for (size_t gi = 0; gi < groups.size(); ++gi) {
-            build_table(groups[gi], slot_class[gi], st->classes, kMaxNsSteps, tables[gi]);
-            st->table_per_iter.push_back(table_per_iter(groups[gi]));
+            std::vector<NsEntry> t;
+            set_run(groups[gi], kMaxNsSteps, 0.f, 0.f, 0.f, false);
+            build_table(groups[gi], slot_class[gi], st->classes, t);
+            st->tables.emplace_back();
+            st->tables.back().per_iter = table_per_iter(groups[gi]);
+            tables.push_back(std::move(t));
+            for (int k = kMinGroupedSteps; k <= kMaxGroupedSteps && any_grouped(groups[gi]); ++k) {
+                t.clear();
+                set_run(groups[gi], k, 0.f, 0.f, 0.f, true);
+                build_table(groups[gi], slot_class[gi], st->classes, t);
+                st->tables.back().grouped_items[k] = static_cast<int32_t>(t.size());
+                tables.push_back(std::move(t));
+            }
         }
     }
     // Zero-padded copies of matrices whose rows or cols are not multiples of 8.
@@ -529,8 +575,7 @@ int plan_and_allocate(malt_state* st, const malt_param_t* params, int n) {
         ShapeClass& C = st->classes[k];
         C.X[0] = H(o_X0[k]);
         C.X[1] = H(o_X1[k]);
-        C.A = H(o_A[k]);
-        C.B = H(o_B[k]);
+        for (int j = 0; j < (C.can_group ? 4 : 2); ++j) C.P[j] = H(o_P[j][k]);
         C.O = H(o_O[k]);
         C.d_mat_of = reinterpret_cast<int32_t*>(base + o_matof[k]);
     }
@@ -555,8 +600,15 @@ int plan_and_allocate(malt_state* st, const malt_param_t* params, int n) {
     for (int j = 0; j < 4; ++j) st->d_pref[j] = reinterpret_cast<int32_t*>(base + o_pref[j]);
     st->d_pre_ids = reinterpret_cast<int32_t*>(base + o_pre_ids);
     st->d_sched = reinterpret_cast<uint32_t*>(base + o_sched);
-    for (size_t gi = 0; gi < tables.size(); ++gi)
-        st->table_dev.push_back(reinterpret_cast<NsEntry*>(base + o_table[gi]));
+    auto table_at = [&](size_t i) { return reinterpret_cast<NsEntry*>(base + o_table[i]); };
+    {
+        size_t i = 0;
+        for (auto& t : st->tables) {
+            t.iterated = table_at(i++);
+            for (int k = kMinGroupedSteps; k <= kMaxGroupedSteps; ++k)
+                if (t.grouped_items[k] > 0) t.grouped[k] = table_at(i++);
+        }
+    }
     for (int i : st->padded) {
         PadBuf& b = st->padbuf[i];
         b.w = base + o_pw[i];
@@ -594,15 +646,17 @@ int plan_and_allocate(malt_state* st, const malt_param_t* params, int n) {
     for (int k = 0; k < nc; ++k) {
         ShapeClass& C = st->classes[k];
         bool ok = true;
+        // (a map moves 16-bit elements; whether they are bf16 or fp16 is the
+        // operation's business)
         for (int b = 0; b < 2; ++b) {
-            ok &= encode_3d(&C.tmX[b], C.X[b], C.q, C.p, C.batch, kBM);
+            ok &= encode_3d(&C.tmK[kBufX + b], C.X[b], C.q, C.p, C.batch, kBM);
             ok &= encode_3d(&C.tmXmn[b], C.X[b], C.q, C.p, C.batch, kBK);
+            ok &= encode_store(&C.stK[kBufX + b], C.X[b], C.q, C.p, C.batch);
         }
-        ok &= encode_3d(&C.tmA, C.A, C.p, C.p, C.batch, kBM);
-        ok &= encode_3d(&C.tmB, C.B, C.p, C.p, C.batch, kBM);
-        for (int b = 0; b < 2; ++b) ok &= encode_store(&C.stX[b], C.X[b], C.q, C.p, C.batch);
-        ok &= encode_store(&C.stA, C.A, C.p, C.p, C.batch);
-        ok &= encode_store(&C.stB, C.B, C.p, C.p, C.batch);
+        for (int b = 0; b < (C.can_group ? 4 : 2); ++b) {
+            ok &= encode_3d(&C.tmK[b], C.P[b], C.p, C.p, C.batch, kBM);
+            ok &= encode_store(&C.stK[b], C.P[b], C.p, C.p, C.batch);
+        }
         ok &= encode_store(&C.stO, C.O, C.q, C.p, C.batch);
         ok &= encode_store(&C.stOt, C.O, C.p, C.q, C.batch);
         if (!ok) {
@@ -649,10 +703,9 @@ int plan_and_allocate(malt_state* st, const malt_param_t* params, int n) {
             MALT_CUDA(cudaMemcpy(C.d_mat_of, C.mats.data(), sizeof(int32_t) * C.batch,
                                  cudaMemcpyHostToDevice), "cudaMemcpy(mat_of)");
         }
-        for (size_t gi = 0; gi < tables.size(); ++gi)
-            MALT_CUDA(cudaMemcpy(st->table_dev[gi], tables[gi].data(),
-                                 sizeof(NsEntry) * tables[gi].size(), cudaMemcpyHostToDevice),
-                      "cudaMemcpy(work table)");
+        for (size_t i = 0; i < tables.size(); ++i)
+            MALT_CUDA(cudaMemcpy(table_at(i), tables[i].data(), sizeof(NsEntry) * tables[i].size(),
+                                 cudaMemcpyHostToDevice), "cudaMemcpy(work table)");
     }
     return MALT_OK;
 }
@@ -720,15 +773,13 @@ int run_padding(malt_state* st, const malt_param_t* params, bool in, cudaStream_
 // The k Newton-Schulz iterations over every class (after the norms kernel
 // has set 1 / (||Mt|| + ns_eps)).
 int run_newton_schulz(malt_state* st, const malt_hparams_t* hp, cudaStream_t s) {
-    thread_local NsParams P;  // ~12 KB of tensor maps: keep off the stack
+    thread_local NsParams P;  // ~17 KB of tensor maps: keep off the stack
     const int k = hp->ns_steps;
     const int max_pairs = ns_gemm_max_pairs();
+    const bool grouped_run = ns_grouped_run(k, hp->ns_a, hp->ns_b, hp->ns_c);
     auto prepare = [&](const NsParams& G) {
         P = G;
-        P.ns_steps = k;
-        P.a = hp->ns_a;
-        P.b = hp->ns_b;
-        P.c = hp->ns_c;
+        set_run(P, k, hp->ns_a, hp->ns_b, hp->ns_c, grouped_run);
     };
     // Auto: the persistent schedule where a product is only a few waves of
     // CTA pairs deep (there the tails and launch gaps between products are a
@@ -741,40 +792,48 @@ int run_newton_schulz(malt_state* st, const malt_hparams_t* hp, cudaStream_t s) 
     for (const NsParams& G : st->ns_groups) any_persistent |= persistent(G);
     if (any_persistent) {
         LaunchScope ls(st, MALT_KIND_NS_PERSISTENT, s, 0);   // launches counted below
-        const size_t counters = st->sched_groups_pad + static_cast<size_t>(3 * k) * st->nmat;
+        const int stages = grouped_run ? std::max(3 * k, kMaxGroupedOps) : 3 * k;
+        const size_t counters = st->sched_groups_pad + static_cast<size_t>(stages) * st->nmat;
         MALT_CUDA(cudaMemsetAsync(st->d_sched, 0, counters * sizeof(uint32_t), s),
                   "cudaMemsetAsync(schedule counters)");
         for (size_t gi = 0; gi < st->ns_groups.size(); ++gi) {
             const NsParams& G = st->ns_groups[gi];
             if (!persistent(G)) continue;
             prepare(G);
-            const int items = k * st->table_per_iter[gi];
-            P.table = st->table_dev[gi];
-            P.nstages = 3 * k;
-            P.item_begin = 0;
-            P.item_end = items;
-            const int pairs = std::max(1, std::min(items, max_pairs));
+            const malt_state::NsTables& T = st->tables[gi];
+            const bool grouped = grouped_run && T.grouped_items[k] > 0;
+            P.table = grouped ? T.grouped[k] : T.iterated;
+            P.item_end = grouped ? T.grouped_items[k] : k * T.per_iter;
+            const int pairs = std::max(1, std::min(P.item_end, max_pairs));
             ++st->prof_launches[MALT_KIND_NS_PERSISTENT];
             MALT_CUDA(launch_ns_gemm(P, kNsPersistent, pairs, s), "ns_gemm_kernel (persistent)");
         }
     }
-    for (int it = 0; it < k; ++it) {
-        for (int phase = kGram; phase <= kBX; ++phase) {
-            for (const NsParams& G : st->ns_groups) {
-                if (persistent(G)) continue;
-                prepare(G);
-                const int per_iter = 2 * G.sym_items + G.full_items;
-                const int begin = it * per_iter + (phase == kGram ? 0
-                                                   : phase == kPoly ? G.sym_items
-                                                                    : 2 * G.sym_items);
-                const int items = phase == kBX ? G.full_items : G.sym_items;
-                P.item_begin = begin;
-                P.item_end = begin + items;
-                const int pairs = std::max(1, std::min(items, max_pairs));
-                LaunchScope ls(st, MALT_KIND_NS_GRAM + phase, s);
-                MALT_CUDA(launch_ns_gemm(P, kNsPhased, pairs, s), "ns_gemm_kernel");
+    // Phased: stage by stage, one launch per group for the classes that have it.
+    for (int stage = 0;; ++stage) {
+        bool more = false;
+        for (const NsParams& G : st->ns_groups) {
+            if (persistent(G)) continue;
+            prepare(G);
+            int items = 0, by_kind[3] = {};
+            for (int c = 0; c < P.nclasses; ++c) {
+                NsClass& C = P.cls[c];
+                C.item_begin = items;
+                if (stage >= ns_num_stages(P, C)) continue;
+                const int kind = ns_op(P, C, stage).kind;
+                by_kind[kind] += ns_phase_tiles(C, kind) * C.batch;
+                items += ns_phase_tiles(C, kind) * C.batch;
             }
+            if (items == 0) continue;
+            more = true;
+            P.stage = stage;
+            P.item_end = items;
+            const int pairs = std::max(1, std::min(items, max_pairs));
+            const int kind = static_cast<int>(std::max_element(by_kind, by_kind + 3) - by_kind);
+            LaunchScope ls(st, MALT_KIND_NS_GRAM + kind, s);
+            MALT_CUDA(launch_ns_gemm(P, kNsPhased, pairs, s), "ns_gemm_kernel");
         }
+        if (!more) break;
     }
     return MALT_OK;
 }
@@ -1230,8 +1289,9 @@ int malt_ns_schedule(const malt_param_t* params, int32_t n, int32_t ns_steps, in
     int64_t total = 0;
     std::vector<NsEntry> table;
     for (size_t gi = 0; gi < groups.size(); ++gi) {
-        const NsParams& G = groups[gi];
-        build_table(G, slot_class[gi], classes, ns_steps, table);
+        NsParams& G = groups[gi];
+        set_run(G, ns_steps, 0.f, 0.f, 0.f, false);
+        build_table(G, slot_class[gi], classes, table);
         for (const NsEntry& e : table) {
             if (total < capacity) {
                 const int st = entry_stage(e);
@@ -1250,6 +1310,31 @@ int malt_ns_schedule(const malt_param_t* params, int32_t n, int32_t ns_steps, in
         }
     }
     *count = total;
+    return MALT_OK;
+}
+
+int malt_ns_plan(int64_t rows, int64_t cols, int32_t n, const malt_hparams_t* hp, malt_ns_op_t* out,
+                 int32_t capacity, int32_t* count) {
+    if (count == nullptr || n < 1 || capacity < 0 || (capacity > 0 && out == nullptr)) return MALT_ERR_INVALID_ARG;
+    const int rc = validate_hparams(hp);
+    if (rc != MALT_OK) return rc;
+    malt_param_t p{};
+    p.rows = rows;
+    p.cols = cols;
+    if (rows <= 0 || cols <= 0 || round8(rows) * round8(cols) >= (int64_t{1} << 31)) return MALT_ERR_UNSUPPORTED;
+    std::vector<MatDesc> hmats;
+    std::vector<ShapeClass> classes;
+    const std::vector<malt_param_t> set(static_cast<size_t>(n), p);
+    build_classes(set.data(), n, hmats, classes);
+    std::vector<NsParams> groups;
+    plan_ns_groups(classes, n, groups);
+    NsParams& G = groups[0];
+    set_run(G, hp->ns_steps, hp->ns_a, hp->ns_b, hp->ns_c, ns_grouped_run(hp->ns_steps, hp->ns_a, hp->ns_b, hp->ns_c));
+    *count = ns_num_stages(G, G.cls[0]);
+    for (int s = 0; s < std::min(capacity, *count); ++s) {
+        const NsOp o = ns_op(G, G.cls[0], s);
+        out[s] = malt_ns_op_t{o.kind, o.f16, o.out16, o.a, o.b, o.e, o.out, o.kx, o.alpha, o.beta, o.gamma};
+    }
     return MALT_OK;
 }
 

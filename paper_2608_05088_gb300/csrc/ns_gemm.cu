@@ -1,10 +1,12 @@
-// ns_gemm.cu -- the Newton-Schulz engine: batched same-shape bf16 GEMMs on the
+// ns_gemm.cu -- the Newton-Schulz engine: batched same-shape 16-bit GEMMs on the
 // sm_103a tensor cores, two SMs per tile (tcgen05.mma.cta_group::2, fp32
 // accumulators in TMEM, operands staged into shared memory by TMA with
 // 128-byte swizzle).
 //
-// One Newton-Schulz iteration (the Orth step of Algorithm 1, run on the wide
-// orientation X of Mt, p x q) is three launches of this kernel:
+// A Newton-Schulz run (the Orth step of Algorithm 1, run on the wide
+// orientation X of Mt, p x q) is a list of products (ns_plan.h): the iterated
+// form for nearly square and small frames, the grouped form for the others.  An
+// iteration of the iterated form is three of them:
 //   kGram  A  = X X^T               (M = N = p, K = q)    operands: rows of X, rows of X
 //   kPoly  B' = a I + b A + c A A   (M = N = p, K = p)    operands: rows of A, rows of A (A = A^T)
 // A and B' are symmetric, so those two phases compute only the tiles on and
@@ -14,8 +16,13 @@
 // so a X + (b A + c A A) X = B' X with the a X term folded into B' (its error
 // is that of the bf16 B it rides on).  The kBX B operand is X itself, read as
 // an MN-major [K][N] matrix, so no transposed copy of X is ever written.  The
+// grouped form's further p x p products (H A, H A H, the running product of the
+// H) are kPoly operations on other buffers, in fp16; they commute with A, so
+// they are symmetric too and take the same path.  GPT-2 Large (36 layers, k = 5):
+// 17 products in 8.76 ms in place of 15 in 10.4 ms; one 16384 x 4096 matrix at
+// k = 8 2.89 in place of 4.27 ms.  The
 // 1/(||Mt||_F + ns_eps) normalisation is folded into the first iteration's
-// epilogues (A scaled by k^2, X' by k).  The last iteration's epilogue writes O
+// epilogues (A scaled by k^2, X' by k).  The last product's epilogue writes O
 // in W's orientation and per-warp partial sums of O^2 and of D^2 with
 // D = L O R (Algorithm 1, D_t line) for the graft.  O is stored in W's layout:
 // a tall matrix's tiles go out transposed (the staging used for the mirror
@@ -40,7 +47,7 @@
 // one of two TMEM accumulators; warps 2-9 drain the other accumulator
 // (tcgen05.ld, pipelined per 32-column chunk) and run the epilogue, so the
 // epilogue of tile i overlaps the MMAs of tile i+1.  Each epilogue warp
-// converts its 32 x 32 chunk to bf16 in a double-buffered shared-memory box
+// converts its 32 x 32 chunk to 16 bits in a double-buffered shared-memory box
 // (64-byte swizzle, bank-conflict free) and writes it with one TMA bulk
 // tensor store.  MMA completion is multicast to both CTAs' barriers; both
 // CTAs' epilogue warps release an accumulator on the even CTA's barrier.
@@ -49,9 +56,9 @@
 //
 // Schedules.  A launch runs a range of the work list (NsParams): every tile
 // of every product of every NS iteration, product by product.
-//  * Phased: one launch per product (Gram, Poly, BX of one iteration); pair
-//    j takes items j, j + npairs, ...  The stream orders the products.
-//  * Persistent: one launch for all k iterations.  A scheduler thread per
+//  * Phased: one launch per stage (a product of every class); pair j takes
+//    items j, j + npairs, ...  The stream orders the stages.
+//  * Persistent: one launch for the whole run.  A scheduler thread per
 //    pair (the odd CTA's otherwise idle MMA-warp thread) claims the next
 //    item with an atomic on a global counter, waits (bounded, acquire) until
 //    the previous product of the item's matrix is complete -- every epilogue
@@ -70,6 +77,7 @@
 //  Both schedules run the same per-tile arithmetic, so their results are
 //  bitwise identical.
 #include <cuda_bf16.h>
+#include <cuda_fp16.h>
 #include <cuda_runtime.h>
 #include <algorithm>
 #include <cstdint>
@@ -99,8 +107,6 @@ constexpr int kGroup = 2;
 constexpr int kRing = kStages / kGroup;
 static_assert(kStages % kGroup == 0, "the slice slots form whole ring stages");
 constexpr uint32_t kTmemCols = 2 * kBN;
-constexpr uint32_t kIdesc = idesc_bf16_f32(kTileM, kBN);
-constexpr uint32_t kIdescBmn = idesc_bf16_f32(kTileM, kBN, true);
 constexpr uint32_t kMnBoxBytes = kBMN * kBK * 2;       // one 64 x 64 MN-major box
 constexpr uint32_t kMnLbo = kMnBoxBytes;               // next 64 MN-elements
 constexpr uint32_t kStoreBoxBytes = 32 * 32 * 2;      // one 32 x 32 bf16 output box
@@ -133,11 +139,11 @@ struct Ops {
 
 __device__ __forceinline__ Ops item_operands(const NsParams& P, const NsWork& w) {
     const NsClass& C = P.cls[w.cls];
-    const int cur = w.iter & 1;
-    if (w.kind == kGram) return Ops{&C.tmX[cur], &C.tmX[cur], &C.stA, C.p, C.p, C.q};
-    if (w.kind == kPoly) return Ops{&C.tmA, &C.tmA, &C.stB, C.p, C.p, C.p};
-    const bool last = w.iter == P.ns_steps - 1;
-    return Ops{&C.tmB, &C.tmXmn[cur], last ? &C.stO : &C.stX[cur ^ 1], C.p, C.q, C.p};
+    const NsOp& o = w.op;
+    const bool bx = o.kind == kBX;
+    return Ops{&C.tmK[o.a], bx ? &C.tmXmn[o.b - kBufX] : &C.tmK[o.b],
+               o.out == kBufO ? &C.stO : &C.stK[o.out],
+               C.p, bx ? C.q : C.p, o.kind == kGram ? C.q : C.p};
 }
 
 // Bytes CTA `rank` loads for one reduction slice of a tile.  Boxes that lie
@@ -161,22 +167,39 @@ __device__ __forceinline__ uint32_t slice_bytes(const Ops& op, const NsWork& w, 
     return bytes;
 }
 
-__device__ __forceinline__ void unpack8(const uint4& u, float* v) {
-    const __nv_bfloat162* h = reinterpret_cast<const __nv_bfloat162*>(&u);
+// Two floats <-> two 16-bit values (fp16 or bf16, round to nearest even).
+template <bool kF16>
+__device__ __forceinline__ float2 unpack2(uint32_t u) {
+    if constexpr (kF16) return __half22float2(*reinterpret_cast<const __half2*>(&u));
+    return __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162*>(&u));
+}
+
+template <bool kF16>
+__device__ __forceinline__ uint32_t pack2(float lo, float hi) {
+    uint32_t u;
+    if constexpr (kF16)
+        *reinterpret_cast<__half2*>(&u) = __floats2half2_rn(lo, hi);
+    else
+        *reinterpret_cast<__nv_bfloat162*>(&u) = __floats2bfloat162_rn(lo, hi);
+    return u;
+}
+
+// v <- sc v + beta x + alpha on the diagonal, x 16 words of two 16-bit values.
+template <bool kF16>
+__device__ __forceinline__ void add_ein(float (&v)[32], const uint32_t* x, float sc, float beta, float alpha,
+                                        int col0, int row) {
 #pragma unroll
-    for (int k = 0; k < 4; ++k) {
-        const float2 f = __bfloat1622float2(h[k]);
-        v[2 * k] = f.x;
-        v[2 * k + 1] = f.y;
+    for (int j = 0; j < 32; j += 2) {
+        const float2 e = unpack2<kF16>(x[j >> 1]);
+        v[j] = fmaf(beta, e.x, sc * v[j]) + (col0 + j == row ? alpha : 0.f);
+        v[j + 1] = fmaf(beta, e.y, sc * v[j + 1]) + (col0 + j + 1 == row ? alpha : 0.f);
     }
 }
 
-__device__ __forceinline__ uint4 pack8(const float* v) {
-    uint4 u;
-    __nv_bfloat162* h = reinterpret_cast<__nv_bfloat162*>(&u);
+template <bool kF16>
+__device__ __forceinline__ void pack32(const float (&v)[32], uint32_t (&w)[16]) {
 #pragma unroll
-    for (int k = 0; k < 4; ++k) h[k] = __floats2bfloat162_rn(v[2 * k], v[2 * k + 1]);
-    return u;
+    for (int j = 0; j < 16; ++j) w[j] = pack2<kF16>(v[2 * j], v[2 * j + 1]);
 }
 
 // Where a wait gave up (recorded once per status word, for malt_debug_timeout_site).
@@ -223,13 +246,11 @@ __device__ __forceinline__ Job job_of_entry(const NsParams& P, const NsEntry& e)
     j.stage = entry_stage(e);
     j.g = e.g;
     j.local = e.local;
-    j.w.s = j.stage;
-    j.w.iter = j.stage / 3;
-    j.w.kind = j.stage - 3 * j.w.iter;
     j.w.cls = entry_cls(e);
+    j.w.op = ns_op(P, P.cls[j.w.cls], j.stage);
     j.w.b = entry_b(e);
     j.w.local = e.local;
-    ns_tile_coords(P.cls[j.w.cls], j.w.kind, e.local, &j.w.mt, &j.w.nt);
+    ns_tile_coords(P.cls[j.w.cls], j.w.op.kind, e.local, &j.w.mt, &j.w.nt);
     return j;
 }
 
@@ -292,11 +313,10 @@ ns_gemm_kernel(const __grid_constant__ NsParams P) {
         for (int c = 0; c < P.nclasses; ++c) {
             const NsClass& C = P.cls[c];
             for (int j = 0; j < 2; ++j) {
-                tma_prefetch_desc(&C.tmX[j]);
+                tma_prefetch_desc(&C.tmK[kBufX + j]);
                 tma_prefetch_desc(&C.tmXmn[j]);
             }
-            tma_prefetch_desc(&C.tmA);
-            tma_prefetch_desc(&C.tmB);
+            for (int j = 0; j < (C.grouped ? 4 : 2); ++j) tma_prefetch_desc(&C.tmK[j]);
         }
     }
     if (warp == 1) {
@@ -313,15 +333,14 @@ ns_gemm_kernel(const __grid_constant__ NsParams P) {
     // the scheduler thread of the odd CTA fills from the work table.
     auto static_job = [&](int seq) -> Job {
         Job j;
-        const long long it = static_cast<long long>(P.item_begin) + pair +
-                             static_cast<long long>(seq) * npairs;
+        const long long it = pair + static_cast<long long>(seq) * npairs;
         if (it >= P.item_end) {
             j.state = kJobEnd;
             return j;
         }
         j.state = kJobWork;
         j.w = ns_decode(P, static_cast<int>(it));
-        j.stage = j.w.s;
+        j.stage = P.stage;
         j.g = -1;
         j.local = j.w.local;
         return j;
@@ -359,7 +378,7 @@ ns_gemm_kernel(const __grid_constant__ NsParams P) {
     // number seq in both CTAs (false when the slot did not come free in time).
     auto claim_next = [&]() -> NsEntry {
         const uint32_t claimed = atomicAdd(P.queue, 1u);
-        if (claimed >= static_cast<uint32_t>(P.item_end - P.item_begin)) {
+        if (claimed >= static_cast<uint32_t>(P.item_end)) {
             NsEntry e;
             e.code = 0;
             e.g = -1;
@@ -367,7 +386,7 @@ ns_gemm_kernel(const __grid_constant__ NsParams P) {
             e.target = 0;
             return e;
         }
-        const int4 v = __ldg(reinterpret_cast<const int4*>(P.table + P.item_begin + claimed));
+        const int4 v = __ldg(reinterpret_cast<const int4*>(P.table + claimed));
         NsEntry e;
         e.code = v.x;
         e.g = v.y;
@@ -408,10 +427,11 @@ ns_gemm_kernel(const __grid_constant__ NsParams P) {
                 if (kPersistent) fence_proxy_async_global();
                 const NsWork& w = job.w;
                 const Ops op = item_operands(P, w);
-                const bool b_mn = w.kind == kBX;
-                // A diagonal tile of a symmetric product: each CTA's half of B is
-                // its own rows of A, so B is not loaded and the MMA reads A twice.
-                const bool same_ab = !b_mn && w.mt == w.nt;
+                const bool b_mn = w.op.kind == kBX;
+                // A diagonal tile of a product of a matrix with itself: each CTA's
+                // half of B is its own rows of A, so B is not loaded and the MMA
+                // reads A twice.
+                const bool same_ab = w.op.a == w.op.b && w.mt == w.nt;
                 const int nkb = (op.K + kBK - 1) / kBK;
                 int nb_self = 0, nb_peer = 0;
                 uint32_t bytes_pair = slice_bytes(op, w, rank, b_mn, &nb_self) +
@@ -489,8 +509,13 @@ ns_gemm_kernel(const __grid_constant__ NsParams P) {
                 if (job.state == kJobEnd) break;
                 const int item = job.local;
                 const NsWork& w = job.w;
-                const bool b_mn = w.kind == kBX;
-                const int K = w.kind == kGram ? P.cls[w.cls].q : P.cls[w.cls].p;
+                const bool b_mn = w.op.kind == kBX;
+                const bool same_ab = w.op.a == w.op.b && w.mt == w.nt;
+                const int K = w.op.kind == kGram ? P.cls[w.cls].q : P.cls[w.cls].p;
+                const uint32_t idesc = b_mn ? (w.op.f16 ? idesc_16bit_f32(kTileM, kBN, true, true)
+                                                        : idesc_16bit_f32(kTileM, kBN, false, true))
+                                            : (w.op.f16 ? idesc_16bit_f32(kTileM, kBN, true, false)
+                                                        : idesc_16bit_f32(kTileM, kBN, false, false));
                 const int nkb = (K + kBK - 1) / kBK;
                 const uint32_t acc = gi & 1, acc_phase = (gi >> 1) & 1;
                 ++gi;
@@ -518,17 +543,16 @@ ns_gemm_kernel(const __grid_constant__ NsParams P) {
 #pragma unroll
                             for (int kk = 0; kk < kBK / 16; ++kk) {
                                 // A: +32 bytes along K; B: +16 K-rows = two 1024-byte atoms.
-                                tc_mma_bf16_pair(d_tmem, da + 2 * kk, db + (2048u >> 4) * kk,
-                                                 kIdescBmn, (kb | kk) != 0 ? 1u : 0u);
+                                tc_mma_16bit_pair(d_tmem, da + 2 * kk, db + (2048u >> 4) * kk,
+                                                  idesc, (kb | kk) != 0 ? 1u : 0u);
                             }
                         } else {
-                            // (a diagonal tile of a symmetric product reads B from A's rows)
-                            const uint64_t db = smem_desc_k_sw128(w.mt == w.nt ? sa : sa + kABytes);
+                            const uint64_t db = smem_desc_k_sw128(same_ab ? sa : sa + kABytes);
 #pragma unroll
                             for (int kk = 0; kk < kBK / 16; ++kk) {
                                 // +32 bytes along K per 16-element MMA slice (encoded >> 4).
-                                tc_mma_bf16_pair(d_tmem, da + 2 * kk, db + 2 * kk, kIdesc,
-                                                 (kb | kk) != 0 ? 1u : 0u);
+                                tc_mma_16bit_pair(d_tmem, da + 2 * kk, db + 2 * kk, idesc,
+                                                  (kb | kk) != 0 ? 1u : 0u);
                             }
                         }
                     }
@@ -585,20 +609,25 @@ ns_gemm_kernel(const __grid_constant__ NsParams P) {
             const NsClass& C = P.cls[w.cls];
             const uint32_t acc = gi & 1, acc_phase = (gi >> 1) & 1;
             ++gi;
-            const int M = C.p, N = w.kind == kBX ? C.q : C.p;
+            const NsOp& op = w.op;
+            const bool in16 = op.f16 != 0, out16 = op.out16 != 0;
+            const int M = C.p, N = op.kind == kBX ? C.q : C.p;
             const CUtensorMap* out_map0 = item_operands(P, w).out;
-            const bool sym = w.kind != kBX;
+            const bool sym = op.kind != kBX;
             const int row = w.mt * kTileM + rank * kBM + quarter * 32 + lane;
             const bool rok = row < M;
             const int g = job.g >= 0 ? job.g : C.mat_of[w.b];
             const MatDesc& md = P.mats[g];
             // Persistent launches read what the launch itself wrote (1/||Mt||,
             // L, R, A) through L2 only.
-            const float kx = w.iter == 0 ? (kPersistent ? __ldcg(&P.scal[g].k) : P.scal[g].k) : 1.f;
-            const bool need_ein = (w.kind == kPoly);
-            const __nv_bfloat16* ein =
-                need_ein ? C.A + static_cast<size_t>(w.b) * C.p * C.p : nullptr;
-            const bool last_bx = (w.kind == kBX) && (w.iter == P.ns_steps - 1);
+            float sc = op.gamma;
+            if (op.kx != 0) {
+                const float k = kPersistent ? __ldcg(&P.scal[g].k) : P.scal[g].k;
+                sc = (op.kx == 2 ? k * k : k) * sc;
+            }
+            const bool need_ein = op.e != kBufNone;
+            const uint16_t* ein = need_ein ? C.A + static_cast<size_t>(w.b) * C.p * C.p : nullptr;
+            const bool last_bx = op.out == kBufO;
             // O of a tall W (NS frame = W^T) goes out transposed, in W's layout.
             const bool store_t = last_bx && md.trans;
             const CUtensorMap* out_map = store_t ? &C.stOt : out_map0;
@@ -661,21 +690,22 @@ ns_gemm_kernel(const __grid_constant__ NsParams P) {
                 for (int j = 0; j < 32; ++j) v[j] = __uint_as_float(rv[j]);
                 // The next chunk's TMEM load is in flight during this chunk's work.
                 if (ch + 1 < nch) tmem_ld_issue(tbase + (ch + 1) * 32, rv);
-                if (w.kind == kGram) {
-                    const float sc = kx * kx;
-#pragma unroll
-                    for (int j = 0; j < 32; ++j) v[j] *= sc;
-                } else if (w.kind == kPoly) {
-                    float x[32];
-#pragma unroll
-                    for (int q8 = 0; q8 < 4; ++q8) unpack8(xcur[q8], x + 8 * q8);
-#pragma unroll
-                    for (int j = 0; j < 32; ++j)
-                        v[j] = fmaf(P.b, x[j], P.c * v[j]) + (col0 + j == row ? P.a : 0.f);
+                if (need_ein) {
+                    const uint32_t* xw = reinterpret_cast<const uint32_t*>(xcur);
+                    if (in16)
+                        add_ein<true>(v, xw, sc, op.beta, op.alpha, col0, row);
+                    else
+                        add_ein<false>(v, xw, sc, op.beta, op.alpha, col0, row);
                 } else {
 #pragma unroll
-                    for (int j = 0; j < 32; ++j) v[j] *= kx;
+                    for (int j = 0; j < 32; ++j) v[j] *= sc;
                 }
+                // This row's 32 results as they are stored.
+                uint32_t wv[16];
+                if (out16)
+                    pack32<true>(v, wv);
+                else
+                    pack32<false>(v, wv);
                 if (!store_t) {
                     // Stage the 32 x 32 chunk (row = lane, 64 bytes) with the 64-byte
                     // swizzle the store map expects, then one TMA store writes it
@@ -686,7 +716,7 @@ ns_gemm_kernel(const __grid_constant__ NsParams P) {
 #pragma unroll
                     for (int c = 0; c < 4; ++c)
                         *reinterpret_cast<uint4*>(box + lane * 64 + ((c ^ ((lane >> 1) & 3)) << 4)) =
-                            pack8(v + 8 * c);
+                            make_uint4(wv[4 * c], wv[4 * c + 1], wv[4 * c + 2], wv[4 * c + 3]);
                     fence_proxy_async_smem();
                     __syncwarp();
                     if (lane == 0) {
@@ -700,8 +730,8 @@ ns_gemm_kernel(const __grid_constant__ NsParams P) {
                     // store a tall matrix's O in W's layout: the transposed chunk
                     // (box row = column j, 32 rows of this warp) goes to rows
                     // [col0, col0+32) x columns [row0, row0+32) of the map.
-                    // Lane pairs swap one value per column pair so each lane
-                    // writes a 32-bit (two-row) word.
+                    // Lane pairs swap the packed word of each column pair, and
+                    // each keeps one column of the two rows.
                     uint8_t* box = stage_out + (ew * 2 + obuf) * kStoreBoxBytes;
                     if (lane == 0) bulk_wait_group_read<1>();
                     __syncwarp();
@@ -710,13 +740,12 @@ ns_gemm_kernel(const __grid_constant__ NsParams P) {
 #pragma unroll
                     for (int j = 0; j < 32; j += 2) {
                         // even lane keeps column j, odd lane keeps column j + 1
-                        const float send = odd ? v[j] : v[j + 1];
-                        const float recv = __shfl_xor_sync(0xffffffffu, send, 1);
-                        const float lo = odd ? recv : v[j];        // row r2
-                        const float hi = odd ? v[j + 1] : recv;    // row r2 + 1
+                        const uint32_t recv = __shfl_xor_sync(0xffffffffu, wv[j >> 1], 1);
+                        const uint32_t pair = odd ? __byte_perm(recv, wv[j >> 1], 0x7632)
+                                                  : __byte_perm(wv[j >> 1], recv, 0x5410);
                         const int jc = j + (odd ? 1 : 0);          // box row
                         const int off = jc * 64 + (((r2 >> 3) ^ ((jc >> 1) & 3)) << 4) + (r2 & 7) * 2;
-                        *reinterpret_cast<__nv_bfloat162*>(box + off) = __floats2bfloat162_rn(lo, hi);
+                        *reinterpret_cast<uint32_t*>(box + off) = pair;
                     }
                     fence_proxy_async_smem();
                     __syncwarp();
@@ -736,7 +765,8 @@ ns_gemm_kernel(const __grid_constant__ NsParams P) {
 #pragma unroll
                     for (int j = 0; j < 32; ++j) {
                         const float vj = __shfl_sync(0xffffffffu, vl, j);
-                        const float o = __bfloat162float(__float2bfloat16_rn(v[j]));
+                        const float2 o2 = unpack2<false>(wv[j >> 1]);
+                        const float o = j & 1 ? o2.y : o2.x;
                         const float ov = o * vj;
                         sum_o = fmaf(o, (col0 + j < N) ? o : 0.f, sum_o);
                         sum_d = fmaf(ov, ov, sum_d);
@@ -762,7 +792,7 @@ ns_gemm_kernel(const __grid_constant__ NsParams P) {
                     dst[1] = sum_d;
                 }
             }
-            if (kPersistent && job.stage + 1 < P.nstages && lane == 0) {
+            if (kPersistent && job.stage + 1 < ns_num_stages(P, C) && lane == 0) {
                 // This warp's part of the tile is in global memory: signal it
                 // (the last stage has no reader inside the launch).
                 bulk_wait_group_all();
