@@ -776,7 +776,9 @@ ns_gemm_kernel(const __grid_constant__ NsParams P) {
             }
             tc_fence_before();
             __syncwarp();
-            if (lane == 0) mbar_arrive_cluster(acc ? tempty_leader1 : tempty_leader0);
+            // The accumulator has been read (the loads have completed and are
+            // ordered by the fence above); no memory contents are handed over.
+            if (lane == 0) mbar_arrive_remote(acc ? tempty_leader1 : tempty_leader0);
             if (last_bx) {
                 if (!rok) sum_o = 0.f;
                 sum_d = rok ? urow * urow * sum_d : 0.f;

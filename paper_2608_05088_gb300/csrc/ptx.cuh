@@ -82,10 +82,12 @@ __device__ __forceinline__ void cluster_sync() {
                  ::: "memory");
 }
 
-// Arrive (release, cluster scope) on an mbarrier given by its shared::cluster address.
-__device__ __forceinline__ void mbar_arrive_cluster(uint32_t cluster_addr) {
-    asm volatile("mbarrier.arrive.release.cluster.shared::cluster.b64 _, [%0];"
-                 ::"r"(cluster_addr) : "memory");
+// Arrive (release at CTA scope, the instruction's default) on an mbarrier of any
+// CTA of the cluster.  For signals that hand over no memory contents (an
+// accumulator that has been read): a release at cluster scope would hold the
+// thread until its earlier loads and stores are performed cluster-wide.
+__device__ __forceinline__ void mbar_arrive_remote(uint32_t cluster_addr) {
+    asm volatile("mbarrier.arrive.shared::cluster.b64 _, [%0];" ::"r"(cluster_addr) : "memory");
 }
 
 // Arrive without release semantics: only the phase count matters (the data
