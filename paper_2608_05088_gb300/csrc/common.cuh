@@ -79,6 +79,12 @@ struct MatScalars {
     float norm_o, norm_d, alpha, nu;
 };
 
+// The step count of a state and what follows from it alone.
+struct StepClock {
+    long long t;    // steps taken (1-based within a step)
+    double bias;    // MALTER: sqrt(1 - mu2^t) / (1 - mu1^t + eps) of this step
+};
+
 struct StepHyper {
     float lr, mu1, mu2, eps, weight_decay;
     float ns_a, ns_b, ns_c, ns_eps;

@@ -42,7 +42,7 @@ cudaError_t launch_pad(const PadParams& P, int32_t blocks, bool in, cudaStream_t
 cudaError_t launch_stats(const MatDesc* mats, const UserPtrs* ptrs, const int32_t* pref,
                          int nmat, int32_t blocks, float mu1, int with_stats, cudaStream_t s);
 cudaError_t launch_finalize(const MatDesc* mats, const UserPtrs* ptrs, const int32_t* pref,
-                            int nmat, int32_t total, float mu2, float eps, long long* tcount,
+                            int nmat, int32_t total, const StepHyper& hp, StepClock* clock,
                             int identity, cudaStream_t s);
 // Prescale: `wide` wide matrices (ids[0 .. wide), wide_blocks blocks) in one
 // launch, then `tall` tall ones (ids[wide ..), tall_blocks blocks) in another;
@@ -52,7 +52,7 @@ cudaError_t launch_prescale(const MatDesc* mats, const UserPtrs* ptrs, const int
                             int32_t tall_blocks, int malter, cudaStream_t s);
 cudaError_t launch_norms(const MatDesc* mats, MatScalars* scal, int nmat, float ns_eps,
                          int malter, cudaStream_t s);
-cudaError_t launch_scalars(const MatDesc* mats, MatScalars* scal, const long long* tcount,
+cudaError_t launch_scalars(const MatDesc* mats, MatScalars* scal, const StepClock* clock,
                            int nmat, const StepHyper& hp, cudaStream_t s);
 cudaError_t launch_apply(const MatDesc* mats, const UserPtrs* ptrs, const MatScalars* scal,
                          const int32_t* pref, int nmat, int32_t blocks, float decay,

@@ -152,7 +152,7 @@ struct malt_state {
     MatDesc* d_mats = nullptr;
     UserPtrs* d_ptrs = nullptr;
     MatScalars* d_scal = nullptr;
-    long long* d_t = nullptr;
+    StepClock* d_clock = nullptr;
     int32_t* d_status = nullptr;
     int32_t* d_pref[4] = {nullptr, nullptr, nullptr, nullptr};  // stats, fin, pre, apply
     int32_t blocks_stats = 0, total_fin = 0, blocks_pre = 0, blocks_apply = 0;
@@ -503,7 +503,7 @@ int plan_and_allocate(malt_state* st, const malt_param_t* params, int n) {
     const size_t o_mats = cv.take(sizeof(MatDesc) * std::max(n, 1));
     const size_t o_ptrs = cv.take(sizeof(UserPtrs) * std::max(n, 1));
     const size_t o_scal = cv.take(sizeof(MatScalars) * std::max(n, 1));
-    const size_t o_t = cv.take(sizeof(long long));
+    const size_t o_t = cv.take(sizeof(StepClock));
     // status word, then the first timeout's site record (site, item, seq, block, thread)
     const size_t o_status = cv.take(sizeof(int32_t) * kStatusWords);
     size_t o_pref[4];
@@ -595,7 +595,7 @@ int plan_and_allocate(malt_state* st, const malt_param_t* params, int n) {
     st->d_mats = reinterpret_cast<MatDesc*>(base + o_mats);
     st->d_ptrs = reinterpret_cast<UserPtrs*>(base + o_ptrs);
     st->d_scal = reinterpret_cast<MatScalars*>(base + o_scal);
-    st->d_t = reinterpret_cast<long long*>(base + o_t);
+    st->d_clock = reinterpret_cast<StepClock*>(base + o_t);
     st->d_status = reinterpret_cast<int32_t*>(base + o_status);
     for (int j = 0; j < 4; ++j) st->d_pref[j] = reinterpret_cast<int32_t*>(base + o_pref[j]);
     st->d_pre_ids = reinterpret_cast<int32_t*>(base + o_pre_ids);
@@ -894,6 +894,7 @@ int run_step(malt_state* st, const malt_param_t* params, int32_t n, const malt_h
         if (rc != MALT_OK) return rc;
     }
     const int nm = st->nmat;
+    const StepHyper sh = step_hyper(hp, malter);
     {
         LaunchScope ls(st, MALT_KIND_STATS, s);
         MALT_CUDA(launch_stats(st->d_mats, st->d_ptrs, st->d_pref[0], nm, st->blocks_stats,
@@ -902,7 +903,7 @@ int run_step(malt_state* st, const malt_param_t* params, int32_t n, const malt_h
     {
         LaunchScope ls(st, MALT_KIND_FINALIZE, s);
         MALT_CUDA(launch_finalize(st->d_mats, st->d_ptrs, st->d_pref[1], nm, st->total_fin,
-                                  hp->mu2, hp->eps, st->d_t, muon, s), "finalize_kernel");
+                                  sh, st->d_clock, muon, s), "finalize_kernel");
     }
     {
         const int wide = st->pre_wide, tall = nm - st->pre_wide;
@@ -919,10 +920,9 @@ int run_step(malt_state* st, const malt_param_t* params, int32_t n, const malt_h
     }
     rc = run_newton_schulz(st, hp, s);
     if (rc != MALT_OK) return rc;
-    const StepHyper sh = step_hyper(hp, malter);
     {
         LaunchScope ls(st, MALT_KIND_SCALARS, s);
-        MALT_CUDA(launch_scalars(st->d_mats, st->d_scal, st->d_t, nm, sh, s), "scalars_kernel");
+        MALT_CUDA(launch_scalars(st->d_mats, st->d_scal, st->d_clock, nm, sh, s), "scalars_kernel");
     }
     if (hooks != nullptr && hooks->wait_before_apply != nullptr)
         MALT_CUDA(cudaStreamWaitEvent(s, hooks->wait_before_apply, 0), "cudaStreamWaitEvent(W read)");
@@ -1107,7 +1107,7 @@ int malt_get_scalars(malt_state_t* st, float* nu_host, int32_t n, int64_t* t_hos
         return MALT_ERR_INVALID_ARG;
     MALT_CUDA(cudaStreamSynchronize(st->last_stream), "cudaStreamSynchronize");
     long long t = 0;
-    MALT_CUDA(cudaMemcpy(&t, st->d_t, sizeof(t), cudaMemcpyDeviceToHost), "cudaMemcpy(t)");
+    MALT_CUDA(cudaMemcpy(&t, &st->d_clock->t, sizeof(t), cudaMemcpyDeviceToHost), "cudaMemcpy(t)");
     *t_host = t;
     if (n > 0) {
         std::vector<MatScalars> s(n);
@@ -1123,7 +1123,7 @@ int malt_set_scalars(malt_state_t* st, const float* nu_host, int32_t n, int64_t 
         return MALT_ERR_INVALID_ARG;
     MALT_CUDA(cudaStreamSynchronize(st->last_stream), "cudaStreamSynchronize");
     const long long t = t_host;
-    MALT_CUDA(cudaMemcpy(st->d_t, &t, sizeof(t), cudaMemcpyHostToDevice), "cudaMemcpy(t)");
+    MALT_CUDA(cudaMemcpy(&st->d_clock->t, &t, sizeof(t), cudaMemcpyHostToDevice), "cudaMemcpy(t)");
     if (n > 0) {
         std::vector<MatScalars> s(n);
         MALT_CUDA(cudaMemcpy(s.data(), st->d_scal, sizeof(MatScalars) * n, cudaMemcpyDeviceToHost),

@@ -55,7 +55,7 @@ float* g_scratch_ptr[kMaxDevices] = {};
 // Momentum update and per-tile partial sums of G^2 (Algorithm 1, M_t / l_t /
 // r_t lines): the statistics block of the step, one kStatRows x kStatCols
 // tile of G per CUDA block.
-__global__ void __launch_bounds__(256)
+__global__ void __launch_bounds__(256, 3)
 noalloc_stats_kernel(const __grid_constant__ MatDesc d, const __grid_constant__ UserPtrs up,
                      float mu1) {
     __shared__ __align__(16) float colsh[8 * malt::kStatCols];

@@ -107,12 +107,14 @@ stats_kernel(const MatDesc* __restrict__ mats, const UserPtrs* __restrict__ ptrs
 __global__ void __launch_bounds__(256)
 finalize_kernel(const MatDesc* __restrict__ mats, const UserPtrs* __restrict__ ptrs,
                 const int32_t* __restrict__ pref, int nmat, int32_t total,
-                float mu2, float eps, long long* tcount, int identity) {
+                StepHyper hp, StepClock* clock, int identity) {
     const int32_t x = blockIdx.x * blockDim.x + threadIdx.x;
-    if (x == 0) *tcount += 1;                 // 1-based step count
+    // (the last thread, which has no entry or a row's short sum)
+    if (blockIdx.x == gridDim.x - 1 && threadIdx.x == blockDim.x - 1)
+        blk::advance_clock(clock, hp.mu1, hp.mu2, hp.eps, hp.malter);
     if (x >= total) return;
     const int g = find_mat(pref, nmat, x);
-    blk::finalize_entry(mats[g], ptrs[g], x - __ldg(pref + g), mu2, eps, identity);
+    blk::finalize_entry(mats[g], ptrs[g], x - __ldg(pref + g), hp.mu2, hp.eps, identity);
 }
 
 // --------------------------------------------------------------- prescale
@@ -156,10 +158,10 @@ norms_kernel(const MatDesc* __restrict__ mats, MatScalars* __restrict__ scal, fl
 // ---------------------------------------------------------------- scalars
 __global__ void __launch_bounds__(blk::kScalarThreads)
 scalars_kernel(const MatDesc* __restrict__ mats, MatScalars* __restrict__ scal,
-               const long long* __restrict__ tcount, StepHyper hp) {
+               const StepClock* __restrict__ clock, StepHyper hp) {
     __shared__ float red[32];
     const int g = blockIdx.x;
-    blk::scalars_matrix(mats[g], scal + g, tcount, hp, threadIdx.x, red);
+    blk::scalars_matrix(mats[g], scal + g, clock, hp, threadIdx.x, red);
 }
 
 // ------------------------------------------------------------------ apply
@@ -231,11 +233,10 @@ cudaError_t launch_stats(const MatDesc* mats, const UserPtrs* ptrs, const int32_
 }
 
 cudaError_t launch_finalize(const MatDesc* mats, const UserPtrs* ptrs, const int32_t* pref,
-                            int nmat, int32_t total, float mu2, float eps, long long* tcount,
+                            int nmat, int32_t total, const StepHyper& hp, StepClock* clock,
                             int identity, cudaStream_t s) {
     const int blocks = (total + 255) / 256 > 0 ? (total + 255) / 256 : 1;
-    finalize_kernel<<<blocks, 256, 0, s>>>(mats, ptrs, pref, nmat, total, mu2, eps, tcount,
-                                          identity);
+    finalize_kernel<<<blocks, 256, 0, s>>>(mats, ptrs, pref, nmat, total, hp, clock, identity);
     return cudaGetLastError();
 }
 
@@ -261,9 +262,9 @@ cudaError_t launch_norms(const MatDesc* mats, MatScalars* scal, int nmat, float 
     return cudaGetLastError();
 }
 
-cudaError_t launch_scalars(const MatDesc* mats, MatScalars* scal, const long long* tcount,
+cudaError_t launch_scalars(const MatDesc* mats, MatScalars* scal, const StepClock* clock,
                            int nmat, const StepHyper& hp, cudaStream_t s) {
-    scalars_kernel<<<nmat, blk::kScalarThreads, 0, s>>>(mats, scal, tcount, hp);
+    scalars_kernel<<<nmat, blk::kScalarThreads, 0, s>>>(mats, scal, clock, hp);
     return cudaGetLastError();
 }
 
