@@ -30,6 +30,7 @@
 #include <nvtx3/nvToolsExt.h>
 
 #include "../../include/malt.h"
+#include "chain.cuh"
 
 namespace {
 
@@ -74,6 +75,7 @@ struct AdamBind {
 // step count t and computes the step's two bias-correction factors once (in
 // double: the update kernel itself does no fp64 arithmetic).
 __global__ void adamw_bind_kernel(const __grid_constant__ AdamBind B, AdamPtrs* __restrict__ table) {
+    malt::chain_wait();
     const int i = threadIdx.x;
     if (i < B.count) table[B.offset + i] = B.p[i];
     if (i == 0 && B.tcount != nullptr) {
@@ -120,7 +122,8 @@ __global__ void __launch_bounds__(kAdamThreads, 6)
 adamw_kernel(const AdamDesc* __restrict__ desc, const AdamPtrs* __restrict__ ptrs,
              const int32_t* __restrict__ pref, int n, const float* __restrict__ factors,
              AdamHyper h) {
-    const int k = find_tensor(pref, n, blockIdx.x);
+    malt::chain_wait();
+    const int k = malt::after_wait(find_tensor(pref, n, blockIdx.x));
     const AdamDesc d = desc[k];
     const AdamPtrs p = ptrs[k];
     const int64_t begin = static_cast<int64_t>(blockIdx.x - __ldg(pref + k)) * kAdamChunk;
@@ -333,14 +336,13 @@ int enqueue_adamw(malt_adamw_state* st, const malt_adamw_param_t* params, int32_
             const malt_adamw_param_t& p = params[off + i];
             B.p[i] = AdamPtrs{p.w, p.w_copy, p.g, p.m, p.v, 1.f - hp->lr * p.weight_decay, 0};
         }
-        adamw_bind_kernel<<<1, kAdamBindChunk, 0, s>>>(B, st->d_ptrs);
-        ADAM_CUDA(cudaGetLastError(), "adamw_bind_kernel");
+        ADAM_CUDA(malt::launch_chained(adamw_bind_kernel, 1, kAdamBindChunk, 0, s, B, st->d_ptrs),
+                  "adamw_bind_kernel");
     }
     if (st->blocks == 0) return MALT_OK;
     const AdamHyper h{hp->lr, hp->beta1, hp->beta2, hp->eps};
-    adamw_kernel<<<st->blocks, kAdamThreads, 0, s>>>(st->d_desc, st->d_ptrs, st->d_pref, n,
-                                                     st->d_factors, h);
-    ADAM_CUDA(cudaGetLastError(), "adamw_kernel");
+    ADAM_CUDA(malt::launch_chained(adamw_kernel, st->blocks, kAdamThreads, 0, s, st->d_desc, st->d_ptrs,
+                                   st->d_pref, n, st->d_factors, h), "adamw_kernel");
     return MALT_OK;
 }
 

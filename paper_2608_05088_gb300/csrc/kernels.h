@@ -50,8 +50,15 @@ cudaError_t launch_finalize(const MatDesc* mats, const UserPtrs* ptrs, const int
 cudaError_t launch_prescale(const MatDesc* mats, const UserPtrs* ptrs, const int32_t* ids,
                             const int32_t* pref, int wide, int32_t wide_blocks, int tall,
                             int32_t tall_blocks, int malter, cudaStream_t s);
+// Counters of the persistent Newton-Schulz launches, zeroed by the norms launch
+// before them: `queues` claim counters and done[stages][nmat] (none: 0 and 0).
+struct SchedCounters {
+    uint32_t* queue;
+    uint32_t* done;
+    int32_t queues, stages;
+};
 cudaError_t launch_norms(const MatDesc* mats, MatScalars* scal, int nmat, float ns_eps,
-                         int malter, cudaStream_t s);
+                         int malter, const SchedCounters& sched, cudaStream_t s);
 cudaError_t launch_scalars(const MatDesc* mats, MatScalars* scal, const StepClock* clock,
                            int nmat, const StepHyper& hp, cudaStream_t s);
 cudaError_t launch_apply(const MatDesc* mats, const UserPtrs* ptrs, const MatScalars* scal,
@@ -69,8 +76,8 @@ cudaError_t launch_guards(void* base, const uint64_t* offsets, int32_t n, bool c
 // CTA pairs (clusters of two).  mode kNsPhased: the items
 // [P.item_begin, P.item_end) of one product, static round-robin.
 // kNsPersistent: the work table P.table, claimed dynamically, each item
-// waiting for its matrix's previous product (P.queue and P.done zeroed before
-// the launch).
+// waiting for its matrix's previous product (P.queue and P.done zeroed by the
+// norms launch).
 cudaError_t launch_ns_gemm(const NsParams& P, int mode, int grid_pairs, cudaStream_t s);
 size_t ns_gemm_smem_bytes();
 int ns_gemm_max_pairs();

@@ -770,6 +770,26 @@ int run_padding(malt_state* st, const malt_param_t* params, bool in, cudaStream_
     return MALT_OK;
 }
 
+// Whether a launch group takes the persistent schedule.  Auto: where a product
+// is only a few waves of CTA pairs deep (there the tails and launch gaps between
+// products are a large share of the time); the phased one where products are deep.
+bool ns_persistent(const malt_state* st, const NsParams& G, int max_pairs) {
+    if (st->ns_schedule != MALT_NS_AUTO) return st->ns_schedule == MALT_NS_PERSISTENT;
+    return G.sym_items < kAutoPersistentWaves * max_pairs;
+}
+
+// The counters that a step's persistent launches use, for the norms launch to zero.
+SchedCounters sched_counters(const malt_state* st, const malt_hparams_t* hp) {
+    const int max_pairs = ns_gemm_max_pairs();
+    SchedCounters c{st->d_sched, st->d_sched + st->sched_groups_pad, 0, 0};
+    for (const NsParams& G : st->ns_groups)
+        if (ns_persistent(st, G, max_pairs)) {
+            c.queues = static_cast<int32_t>(st->ns_groups.size());
+            c.stages = std::max(3 * hp->ns_steps, hp->ns_steps <= kMaxGroupedSteps ? kMaxGroupedOps : 0);
+        }
+    return c;
+}
+
 // The k Newton-Schulz iterations over every class (after the norms kernel
 // has set 1 / (||Mt|| + ns_eps)).
 int run_newton_schulz(malt_state* st, const malt_hparams_t* hp, cudaStream_t s) {
@@ -781,24 +801,13 @@ int run_newton_schulz(malt_state* st, const malt_hparams_t* hp, cudaStream_t s) 
         P = G;
         set_run(P, k, hp->ns_a, hp->ns_b, hp->ns_c, grouped_run);
     };
-    // Auto: the persistent schedule where a product is only a few waves of
-    // CTA pairs deep (there the tails and launch gaps between products are a
-    // large share of the time), the phased one where products are deep.
-    auto persistent = [&](const NsParams& G) {
-        if (st->ns_schedule != MALT_NS_AUTO) return st->ns_schedule == MALT_NS_PERSISTENT;
-        return G.sym_items < kAutoPersistentWaves * max_pairs;
-    };
     bool any_persistent = false;
-    for (const NsParams& G : st->ns_groups) any_persistent |= persistent(G);
+    for (const NsParams& G : st->ns_groups) any_persistent |= ns_persistent(st, G, max_pairs);
     if (any_persistent) {
         LaunchScope ls(st, MALT_KIND_NS_PERSISTENT, s, 0);   // launches counted below
-        const int stages = grouped_run ? std::max(3 * k, kMaxGroupedOps) : 3 * k;
-        const size_t counters = st->sched_groups_pad + static_cast<size_t>(stages) * st->nmat;
-        MALT_CUDA(cudaMemsetAsync(st->d_sched, 0, counters * sizeof(uint32_t), s),
-                  "cudaMemsetAsync(schedule counters)");
         for (size_t gi = 0; gi < st->ns_groups.size(); ++gi) {
             const NsParams& G = st->ns_groups[gi];
-            if (!persistent(G)) continue;
+            if (!ns_persistent(st, G, max_pairs)) continue;
             prepare(G);
             const malt_state::NsTables& T = st->tables[gi];
             const bool grouped = grouped_run && T.grouped_items[k] > 0;
@@ -813,7 +822,7 @@ int run_newton_schulz(malt_state* st, const malt_hparams_t* hp, cudaStream_t s) 
     for (int stage = 0;; ++stage) {
         bool more = false;
         for (const NsParams& G : st->ns_groups) {
-            if (persistent(G)) continue;
+            if (ns_persistent(st, G, max_pairs)) continue;
             prepare(G);
             int items = 0, by_kind[3] = {};
             for (int c = 0; c < P.nclasses; ++c) {
@@ -916,7 +925,8 @@ int run_step(malt_state* st, const malt_param_t* params, int32_t n, const malt_h
         MALT_CUDA(cudaEventRecord(hooks->record_g_consumed, s), "cudaEventRecord(G consumed)");
     {
         LaunchScope ls(st, MALT_KIND_NORMS, s);
-        MALT_CUDA(launch_norms(st->d_mats, st->d_scal, nm, hp->ns_eps, malter, s), "norms_kernel");
+        MALT_CUDA(launch_norms(st->d_mats, st->d_scal, nm, hp->ns_eps, malter, sched_counters(st, hp), s),
+                  "norms_kernel");
     }
     rc = run_newton_schulz(st, hp, s);
     if (rc != MALT_OK) return rc;

@@ -34,6 +34,7 @@
 #include <mutex>
 
 #include "../../include/malt.h"
+#include "chain.cuh"
 #include "common.cuh"
 #include "stream_blocks.cuh"
 
@@ -59,6 +60,7 @@ __global__ void __launch_bounds__(256, 3)
 noalloc_stats_kernel(const __grid_constant__ MatDesc d, const __grid_constant__ UserPtrs up,
                      float mu1) {
     __shared__ __align__(16) float colsh[8 * malt::kStatCols];
+    malt::chain_wait();
     malt::blk::stats_block<true>(d, up, blockIdx.x, mu1, threadIdx.x, colsh);
 }
 
@@ -68,6 +70,7 @@ noalloc_stats_kernel(const __grid_constant__ MatDesc d, const __grid_constant__ 
 __global__ void __launch_bounds__(256)
 noalloc_finalize_kernel(const __grid_constant__ MatDesc d, const __grid_constant__ UserPtrs up,
                         float mu2, float eps) {
+    malt::chain_wait();
     const int x = blockIdx.x * blockDim.x + threadIdx.x;
     if (x < d.m + d.n) malt::blk::finalize_entry(d, up, x, mu2, eps, 0);
 }
@@ -145,12 +148,11 @@ extern "C" int malt_stats_noalloc(const void* g, int32_t g_dtype, float* m, floa
     d.R = R_out;
     const UserPtrs up{nullptr, g, m, l, r, nullptr};
     cudaStream_t s = static_cast<cudaStream_t>(stream);
-    noalloc_stats_kernel<<<static_cast<unsigned>(cb_count * rb_count), 256, 0, s>>>(d, up, mu1);
-    cudaError_t e = cudaGetLastError();
+    cudaError_t e = malt::launch_chained(noalloc_stats_kernel, static_cast<unsigned>(cb_count * rb_count), 256,
+                                         0, s, d, up, mu1);
     if (e == cudaSuccess) {
-        noalloc_finalize_kernel<<<static_cast<unsigned>((rows + cols + 255) / 256), 256, 0, s>>>(
-            d, up, mu2, eps);
-        e = cudaGetLastError();
+        e = malt::launch_chained(noalloc_finalize_kernel, static_cast<unsigned>((rows + cols + 255) / 256), 256,
+                                 0, s, d, up, mu2, eps);
     }
     if (e != cudaSuccess) {
         std::fprintf(stderr, "malt_stats_noalloc: launch failed: %s\n", cudaGetErrorString(e));

@@ -84,6 +84,7 @@
 #include <cstdio>
 #include <mutex>
 
+#include "chain.cuh"
 #include "common.cuh"
 #include "kernels.h"
 #include "ptx.cuh"
@@ -323,6 +324,8 @@ ns_gemm_kernel(const __grid_constant__ NsParams P) {
         tmem_alloc_pair(&tmem_slot, kTmemCols);
         tmem_relinquish_pair();
     }
+    // What precedes touches no global memory that an earlier launch writes.
+    chain_wait();
     tc_fence_before();
     cluster_sync();          // both CTAs' barriers initialised, TMEM allocated
     tc_fence_after();
@@ -890,11 +893,9 @@ cudaError_t ns_gemm_configure() {
 cudaError_t launch_ns_gemm(const NsParams& P, int mode, int grid_pairs, cudaStream_t s) {
     const cudaError_t ce = ns_gemm_configure();
     if (ce != cudaSuccess) return ce;
-    if (mode == kNsPersistent)
-        ns_gemm_kernel<kNsPersistent><<<2 * grid_pairs, kThreads, kSmemBytes, s>>>(P);
-    else
-        ns_gemm_kernel<kNsPhased><<<2 * grid_pairs, kThreads, kSmemBytes, s>>>(P);
-    const cudaError_t e = cudaGetLastError();
+    const cudaError_t e = launch_chained(mode == kNsPersistent ? ns_gemm_kernel<kNsPersistent>
+                                                               : ns_gemm_kernel<kNsPhased>,
+                                         2 * grid_pairs, kThreads, kSmemBytes, s, P);
     if (e != cudaSuccess) {
         cudaFuncAttributes fa{};
         if (mode == kNsPersistent)

@@ -9,6 +9,7 @@
 #include <cuda_runtime.h>
 #include <cstdint>
 
+#include "chain.cuh"
 #include "common.cuh"
 #include "kernels.h"
 #include "ptx.cuh"
@@ -31,6 +32,7 @@ __device__ __forceinline__ int find_mat(const int32_t* __restrict__ pref, int nm
 
 // ---------------------------------------------------------------- binding
 __global__ void bind_kernel(const __grid_constant__ BindParams P, UserPtrs* __restrict__ table) {
+    chain_wait();
     const int i = threadIdx.x;
     if (i < P.count) table[P.offset + i] = P.p[i];
 }
@@ -46,6 +48,7 @@ __device__ __forceinline__ void copy_row(const T* __restrict__ src, T* __restric
 
 template <bool kIn>
 __global__ void __launch_bounds__(256) pad_kernel(const __grid_constant__ PadParams P) {
+    chain_wait();
     int k = 0;
     while (k + 1 < P.count && P.e[k + 1].block_begin <= static_cast<int32_t>(blockIdx.x)) ++k;
     const PadEntry& e = P.e[k];
@@ -98,7 +101,8 @@ __global__ void __launch_bounds__(256, 3)
 stats_kernel(const MatDesc* __restrict__ mats, const UserPtrs* __restrict__ ptrs,
              const int32_t* __restrict__ pref, int nmat, float mu1) {
     __shared__ __align__(16) float colsh[8 * kStatCols];
-    const int g = find_mat(pref, nmat, blockIdx.x);
+    chain_wait();
+    const int g = after_wait(find_mat(pref, nmat, blockIdx.x));
     blk::stats_block<kStats>(mats[g], ptrs[g], blockIdx.x - __ldg(pref + g), mu1, threadIdx.x,
                              colsh);
 }
@@ -108,12 +112,13 @@ __global__ void __launch_bounds__(256)
 finalize_kernel(const MatDesc* __restrict__ mats, const UserPtrs* __restrict__ ptrs,
                 const int32_t* __restrict__ pref, int nmat, int32_t total,
                 StepHyper hp, StepClock* clock, int identity) {
+    chain_wait();
     const int32_t x = blockIdx.x * blockDim.x + threadIdx.x;
     // (the last thread, which has no entry or a row's short sum)
     if (blockIdx.x == gridDim.x - 1 && threadIdx.x == blockDim.x - 1)
         blk::advance_clock(clock, hp.mu1, hp.mu2, hp.eps, hp.malter);
     if (x >= total) return;
-    const int g = find_mat(pref, nmat, x);
+    const int g = after_wait(find_mat(pref, nmat, x));
     blk::finalize_entry(mats[g], ptrs[g], x - __ldg(pref + g), hp.mu2, hp.eps, identity);
 }
 
@@ -126,9 +131,10 @@ prescale_wide_kernel(const MatDesc* __restrict__ mats, const UserPtrs* __restric
                      const int32_t* __restrict__ ids, const int32_t* __restrict__ pref, int count,
                      int malter) {
     __shared__ float2 red[8];
+    chain_wait();
     const int32_t x = blockIdx.x;
     const int k = find_mat(pref, count, x);
-    const int g = __ldg(ids + k);
+    const int g = after_wait(__ldg(ids + k));
     blk::prescale_block<false>(mats[g], ptrs[g], x - __ldg(pref + k), malter, threadIdx.x, nullptr,
                                red);
 }
@@ -139,9 +145,10 @@ prescale_tall_kernel(const MatDesc* __restrict__ mats, const UserPtrs* __restric
                      int32_t base, int malter) {
     __shared__ __align__(16) float tile[blk::kPreTileFloats];
     __shared__ float2 red[8];
+    chain_wait();
     const int32_t x = base + static_cast<int32_t>(blockIdx.x);   // pref continues the wide launch's
     const int k = find_mat(pref, count, x);
-    const int g = __ldg(ids + k);
+    const int g = after_wait(__ldg(ids + k));
     blk::prescale_block<true>(mats[g], ptrs[g], x - __ldg(pref + k), malter, threadIdx.x, tile,
                               red);
 }
@@ -149,9 +156,14 @@ prescale_tall_kernel(const MatDesc* __restrict__ mats, const UserPtrs* __restric
 // ------------------------------------------------------------------ norms
 __global__ void __launch_bounds__(256)
 norms_kernel(const MatDesc* __restrict__ mats, MatScalars* __restrict__ scal, float ns_eps,
-             int malter) {
+             int malter, SchedCounters sched) {
     __shared__ float red[32];
-    const int g = blockIdx.x;
+    chain_wait();
+    const int g = after_wait(static_cast<int>(blockIdx.x));
+    // The persistent Newton-Schulz launches that follow count from zero.
+    for (int s = threadIdx.x; s < sched.stages; s += blockDim.x)
+        sched.done[static_cast<size_t>(s) * gridDim.x + g] = 0;
+    for (int i = threadIdx.x; g == 0 && i < sched.queues; i += blockDim.x) sched.queue[i] = 0;
     blk::norms_matrix(mats[g], scal + g, ns_eps, malter, threadIdx.x, red);
 }
 
@@ -160,7 +172,8 @@ __global__ void __launch_bounds__(blk::kScalarThreads)
 scalars_kernel(const MatDesc* __restrict__ mats, MatScalars* __restrict__ scal,
                const StepClock* __restrict__ clock, StepHyper hp) {
     __shared__ float red[32];
-    const int g = blockIdx.x;
+    chain_wait();
+    const int g = after_wait(static_cast<int>(blockIdx.x));
     blk::scalars_matrix(mats[g], scal + g, clock, hp, threadIdx.x, red);
 }
 
@@ -169,7 +182,8 @@ __global__ void __launch_bounds__(256, 8)
 apply_kernel(const MatDesc* __restrict__ mats, const UserPtrs* __restrict__ ptrs,
              const MatScalars* __restrict__ scal, const int32_t* __restrict__ pref, int nmat,
              float decay) {
-    const int g = find_mat(pref, nmat, blockIdx.x);
+    chain_wait();
+    const int g = after_wait(find_mat(pref, nmat, blockIdx.x));
     blk::apply_block(mats[g], ptrs[g], blockIdx.x - __ldg(pref + g), scal[g].scale, decay,
                      threadIdx.x);
 }
@@ -211,70 +225,56 @@ __global__ void guard_kernel(uint8_t* base, const uint64_t* __restrict__ offsets
 
 // ------------------------------------------------------------------ launch
 cudaError_t launch_bind(const BindParams& P, UserPtrs* table, cudaStream_t s) {
-    bind_kernel<<<1, kBindChunk, 0, s>>>(P, table);
-    return cudaGetLastError();
+    return launch_chained(bind_kernel, 1, kBindChunk, 0, s, P, table);
 }
 
 cudaError_t launch_pad(const PadParams& P, int32_t blocks, bool in, cudaStream_t s) {
-    if (in)
-        pad_kernel<true><<<blocks, 256, 0, s>>>(P);
-    else
-        pad_kernel<false><<<blocks, 256, 0, s>>>(P);
-    return cudaGetLastError();
+    return launch_chained(in ? pad_kernel<true> : pad_kernel<false>, blocks, 256, 0, s, P);
 }
 
 cudaError_t launch_stats(const MatDesc* mats, const UserPtrs* ptrs, const int32_t* pref,
                          int nmat, int32_t blocks, float mu1, int with_stats, cudaStream_t s) {
-    if (with_stats)
-        stats_kernel<true><<<blocks, 256, 0, s>>>(mats, ptrs, pref, nmat, mu1);
-    else
-        stats_kernel<false><<<blocks, 256, 0, s>>>(mats, ptrs, pref, nmat, mu1);
-    return cudaGetLastError();
+    return launch_chained(with_stats ? stats_kernel<true> : stats_kernel<false>, blocks, 256, 0, s,
+                          mats, ptrs, pref, nmat, mu1);
 }
 
 cudaError_t launch_finalize(const MatDesc* mats, const UserPtrs* ptrs, const int32_t* pref,
                             int nmat, int32_t total, const StepHyper& hp, StepClock* clock,
                             int identity, cudaStream_t s) {
     const int blocks = (total + 255) / 256 > 0 ? (total + 255) / 256 : 1;
-    finalize_kernel<<<blocks, 256, 0, s>>>(mats, ptrs, pref, nmat, total, hp, clock, identity);
-    return cudaGetLastError();
+    return launch_chained(finalize_kernel, blocks, 256, 0, s, mats, ptrs, pref, nmat, total, hp, clock,
+                          identity);
 }
 
 cudaError_t launch_prescale(const MatDesc* mats, const UserPtrs* ptrs, const int32_t* ids,
                             const int32_t* pref, int wide, int32_t wide_blocks, int tall,
                             int32_t tall_blocks, int malter, cudaStream_t s) {
     if (wide > 0 && wide_blocks > 0) {
-        prescale_wide_kernel<<<wide_blocks, 256, 0, s>>>(mats, ptrs, ids, pref, wide, malter);
-        const cudaError_t e = cudaGetLastError();
+        const cudaError_t e = launch_chained(prescale_wide_kernel, wide_blocks, 256, 0, s, mats, ptrs, ids,
+                                             pref, wide, malter);
         if (e != cudaSuccess) return e;
     }
-    if (tall > 0 && tall_blocks > 0) {
-        prescale_tall_kernel<<<tall_blocks, 256, 0, s>>>(mats, ptrs, ids + wide, pref + wide, tall,
-                                                         wide_blocks, malter);
-        return cudaGetLastError();
-    }
+    if (tall > 0 && tall_blocks > 0)
+        return launch_chained(prescale_tall_kernel, tall_blocks, 256, 0, s, mats, ptrs, ids + wide,
+                              pref + wide, tall, wide_blocks, malter);
     return cudaSuccess;
 }
 
 cudaError_t launch_norms(const MatDesc* mats, MatScalars* scal, int nmat, float ns_eps,
-                         int malter, cudaStream_t s) {
-    norms_kernel<<<nmat, 256, 0, s>>>(mats, scal, ns_eps, malter);
-    return cudaGetLastError();
+                         int malter, const SchedCounters& sched, cudaStream_t s) {
+    return launch_chained(norms_kernel, nmat, 256, 0, s, mats, scal, ns_eps, malter, sched);
 }
 
 cudaError_t launch_scalars(const MatDesc* mats, MatScalars* scal, const StepClock* clock,
                            int nmat, const StepHyper& hp, cudaStream_t s) {
-    scalars_kernel<<<nmat, blk::kScalarThreads, 0, s>>>(mats, scal, clock, hp);
-    return cudaGetLastError();
+    return launch_chained(scalars_kernel, nmat, blk::kScalarThreads, 0, s, mats, scal, clock, hp);
 }
 
 cudaError_t launch_apply(const MatDesc* mats, const UserPtrs* ptrs, const MatScalars* scal,
                          const int32_t* pref, int nmat, int32_t blocks, float decay,
                          cudaStream_t s) {
-    apply_kernel<<<blocks, 256, 0, s>>>(mats, ptrs, scal, pref, nmat, decay);
-    return cudaGetLastError();
+    return launch_chained(apply_kernel, blocks, 256, 0, s, mats, ptrs, scal, pref, nmat, decay);
 }
-
 
 cudaError_t launch_guards(void* base, const uint64_t* offsets, int32_t n, bool check,
                           unsigned long long* bad, cudaStream_t s) {
