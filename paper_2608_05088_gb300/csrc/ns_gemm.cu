@@ -58,22 +58,21 @@
 // of every product of every NS iteration, product by product.
 //  * Phased: one launch per stage (a product of every class); pair j takes
 //    items j, j + npairs, ...  The stream orders the stages.
-//  * Persistent: one launch for the whole run.  A scheduler thread per
-//    pair (the odd CTA's otherwise idle MMA-warp thread) claims the next
-//    item with an atomic on a global counter, waits (bounded, acquire) until
-//    the previous product of the item's matrix is complete -- every epilogue
-//    warp of every tile of that product has signalled done[] after its TMA
-//    stores completed -- and publishes the item to a 4-slot ring in both
-//    CTAs' shared memory (st.async messages on mbarriers), a few items ahead
-//    of the producers, MMA and epilogues that read it.  Each product of a
-//    matrix depends only on the previous product of the same matrix, so
-//    tiles of the next product of one matrix start while the current
+//  * Persistent: one launch for the whole run.  A scheduler thread per pair (the
+//    odd CTA's otherwise idle MMA-warp thread) claims items with an atomic on a
+//    global counter and publishes them to a 4-slot ring in both CTAs' shared
+//    memory (st.async messages on mbarriers).  Before it reads a tile's
+//    operands, each producer waits (bounded, acquire) until the previous stage
+//    of the tile's matrix is complete -- every epilogue warp of every tile of
+//    that stage has signalled done[] after its TMA stores completed.  Each
+//    product of a matrix depends only on the previous products of the same
+//    matrix, so tiles of the next product of one matrix start while the current
 //    product of another matrix is still running: no grid-wide barrier
 //    between products, no launch gaps, no wave tails except the last.
-//    Items are claimed in list order by running CTAs only, so every item a
-//    tile waits for is held by a CTA that is running and whose own
-//    dependencies come earlier still: the schedule cannot deadlock, whatever
-//    number of CTA pairs is resident.
+//    Items are claimed in list order by running CTAs only and each pair runs its
+//    items in order, so every item a tile waits for is held by a CTA that is
+//    running and whose own dependencies come earlier still: the schedule cannot
+//    deadlock, whatever number of CTA pairs is resident.
 //  Both schedules run the same per-tile arithmetic, so their results are
 //  bitwise identical.
 #include <cuda_bf16.h>
@@ -94,7 +93,8 @@ namespace malt {
 namespace {
 
 constexpr int kEpiWarps = kEpiWarpsPerCta;
-constexpr int kThreads = 64 + 32 * kEpiWarps;
+// A persistent launch has one more warp, which signals finished tiles.
+constexpr int ns_threads(int mode) { return 64 + 32 * kEpiWarps + (mode == kNsPersistent ? 32 : 0); }
 constexpr int kEpiCols = kBN / (kEpiWarps / 4);        // accumulator columns per warp
 constexpr int kEpiChunks = kEpiCols / 32;
 constexpr int kHalfN = kBN / 2;                        // B rows (or columns) per CTA
@@ -120,9 +120,13 @@ constexpr uint16_t kPairMask = 0x3;
 // both producers, the even CTA's MMA thread, every epilogue warp of both CTAs.
 constexpr int kItemSlots = 4;
 constexpr int kNoItem = -0x7fffffff;   // never stored in the ring
-constexpr uint32_t kItemReaders = 3 + 2 * kEpiWarps;
+constexpr uint32_t kItemReaders = 5 + 2 * kEpiWarps;
 static_assert(2 * kEpiWarps == static_cast<int>(kNsSignalsPerTile),
-              "every epilogue warp of the pair signals a finished tile once");
+              "a finished tile counts one signal per epilogue warp of the pair");
+// Signalled tiles whose stores the epilogue warps may still be reporting: a
+// warp reaches tile i + 4 only after every warp has released the accumulator
+// of tile i + 2, that is, has reported tile i.
+constexpr int kSigSlots = 4;
 
 static_assert(kBK * 2 == 128, "one K slice must be one 128-byte swizzle row");
 static_assert(kTmemCols <= 512, "two accumulators must fit in TMEM");
@@ -206,12 +210,13 @@ __device__ __forceinline__ void pack32(const float (&v)[32], uint32_t (&w)[16]) 
 // Where a wait gave up (recorded once per status word, for malt_debug_timeout_site).
 enum WaitSite : int32_t {
     kSiteClaim = 1,      // scheduler: a ring slot to become free
-    kSiteDepLoad = 2,    // scheduler: the previous product of the item's matrix
+    kSiteDepLoad = 2,    // the previous stage of the matrix (producer; + 16 scheduler; + 32 epilogue)
     kSiteStage = 3,      // producer: a free operand stage
     kSiteItem = 4,       // ring reader: the next item (+ 16 * role)
     kSiteAccFree = 5,    // MMA: a free accumulator
     kSiteStageFull = 6,  // MMA: operands of a stage
     kSiteAccFull = 7,    // epilogue: a finished accumulator
+    kSiteSignal = 8,     // signal warp: the epilogue warps' stores of a tile
     kSiteDrain = 9,      // MMA: the last MMAs before TMEM is freed
 };
 
@@ -234,6 +239,7 @@ struct Job {
     int32_t stage;    // stage of the work table (persistent) or product index (phased)
     int32_t g;        // matrix (-1 when not known yet: phased)
     int32_t local;
+    uint32_t target;  // signals that the matrix's previous stage must have (0: none)
     NsWork w;
 };
 
@@ -247,6 +253,7 @@ __device__ __forceinline__ Job job_of_entry(const NsParams& P, const NsEntry& e)
     j.stage = entry_stage(e);
     j.g = e.g;
     j.local = e.local;
+    j.target = e.target;
     j.w.cls = entry_cls(e);
     j.w.op = ns_op(P, P.cls[j.w.cls], j.stage);
     j.w.b = entry_b(e);
@@ -258,7 +265,7 @@ __device__ __forceinline__ Job job_of_entry(const NsParams& P, const NsEntry& e)
 }  // namespace
 
 template <int kMode>
-__global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
+__global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(ns_threads(kMode), 1)
 ns_gemm_kernel(const __grid_constant__ NsParams P) {
     constexpr bool kPersistent = kMode == kNsPersistent;   // table-driven, claimed dynamically
     extern __shared__ uint8_t smem_raw[];
@@ -270,6 +277,7 @@ ns_gemm_kernel(const __grid_constant__ NsParams P) {
     __shared__ __align__(8) uint64_t item_full[kItemSlots];
     __shared__ __align__(8) uint64_t item_empty[kItemSlots];
     __shared__ NsEntry item_ring[kItemSlots];
+    __shared__ __align__(8) uint64_t sig_bar[kSigSlots];
     __shared__ uint32_t tmem_slot;
     __shared__ int abort_sh;
     volatile int* abort_flag = &abort_sh;
@@ -305,6 +313,7 @@ ns_gemm_kernel(const __grid_constant__ NsParams P) {
                 mbar_init(&item_full[s], 1);
                 mbar_init(&item_empty[s], kItemReaders);
             }
+            for (int s = 0; s < kSigSlots; ++s) mbar_init(&sig_bar[s], kEpiWarps);
         }
         abort_sh = 0;
         fence_barrier_init();
@@ -346,6 +355,7 @@ ns_gemm_kernel(const __grid_constant__ NsParams P) {
         j.stage = P.stage;
         j.g = -1;
         j.local = j.w.local;
+        j.target = 0;
         return j;
     };
     // The ring entry of sequence number seq (false when the wait gave up).
@@ -403,8 +413,8 @@ ns_gemm_kernel(const __grid_constant__ NsParams P) {
         if (!mbar_wait_cluster_bounded(&item_empty[slot], par ^ 1u, budget, abort_flag)) return false;
         // The entry travels as an asynchronous store that completes on the
         // slot's full barrier in each CTA.  The arrive releases at cluster
-        // scope what this thread acquired from the dependency counter, so a
-        // reader that sees the item also sees the data the item reads.
+        // scope what this thread may have acquired from the dependency counter,
+        // so a reader of an item without a target sees the data the item reads.
         for (uint32_t r = 0; r < 2; ++r) {
             const uint32_t bar = mapa_shared(smem_u32(&item_full[slot]), r);
             mbar_arrive_expect_tx_cluster(bar, 16u);
@@ -412,6 +422,16 @@ ns_gemm_kernel(const __grid_constant__ NsParams P) {
                         static_cast<int32_t>(e.target), bar);
         }
         return true;
+    };
+
+    // Wait (bounded, acquire) until the previous stage of the job's matrix is
+    // stored.  Each reader of another CTA's results waits for itself, with the
+    // item already decoded: handed on by the scheduler only once the stage was
+    // complete, an item reached the producers 1.2 us later (one 256 x 512 matrix
+    // has 15 such waits in a row).
+    auto stage_done = [&](int stage, int g, uint32_t target) -> bool {
+        return target == 0 || counter_wait_bounded(P.done + (stage - 1) * P.nmat + g, target, budget, P.status,
+                                                   kStatusTimeout, abort_flag);
     };
 
     if (warp == 0) {
@@ -426,8 +446,15 @@ ns_gemm_kernel(const __grid_constant__ NsParams P) {
                 }
                 if (job.state == kJobEnd) break;
                 const int item = job.local;
-                // The loads below read what other CTAs stored in this launch.
-                if (kPersistent) fence_proxy_async_global();
+                // The loads below read what other CTAs stored in this launch: wait
+                // for the previous stage of this matrix.
+                if (kPersistent) {
+                    if (!stage_done(job.stage, job.g, job.target)) {
+                        raise_timeout(P, abort_flag, kSiteDepLoad, item, seq);
+                        break;
+                    }
+                    fence_proxy_async_global();
+                }
                 const NsWork& w = job.w;
                 const Ops op = item_operands(P, w);
                 const bool b_mn = w.op.kind == kBX;
@@ -478,25 +505,27 @@ ns_gemm_kernel(const __grid_constant__ NsParams P) {
     } else if (warp == 1) {
         if (kPersistent && lane == 0 && !leader) {
             // ------------------------------------------ scheduler (odd CTA)
-            // Claim items in table order, one ahead; publish each once the
-            // previous stage of its matrix is complete, up to kItemSlots
-            // ahead of the slowest reader.  Waiting here keeps the acquire
-            // round trip off the producers' path.
-            NsEntry next = claim_next();
+            // Claim items in table order and publish them up to kItemSlots ahead
+            // of the slowest reader.  The next item is claimed only once the
+            // last one can run: claimed at once, five items a pair left a stage
+            // of 136 tiles to 28 of the 76 pairs (one 4096 x 4096 matrix 916 us
+            // -> 1245).
             for (int seq = 0;; ++seq) {
-                const NsEntry e = next;
-                if (e.g >= 0 && e.target > 0 &&
-                    !counter_wait_bounded(P.done + (entry_stage(e) - 1) * P.nmat + e.g, e.target,
-                                          P.budget_ns, P.status, kStatusTimeout, abort_flag)) {
-                    raise_timeout(P, abort_flag, kSiteDepLoad, e.local, seq);
-                    break;
-                }
+                NsEntry e = claim_next();
+                const uint32_t target = e.target;
+                // (complete already: the readers need not look again)
+                if (e.g >= 0 && target > 0 &&
+                    ld_acquire_gpu(P.done + (entry_stage(e) - 1) * P.nmat + e.g) >= target)
+                    e.target = 0;
                 if (!publish_item(seq, e)) {
                     raise_timeout(P, abort_flag, kSiteClaim, e.local, seq);
                     break;
                 }
                 if (e.g < 0) break;
-                next = claim_next();
+                if (e.target > 0 && !stage_done(entry_stage(e), e.g, target)) {
+                    raise_timeout(P, abort_flag, kSiteDepLoad + 16, e.local, seq);
+                    break;
+                }
             }
         }
         // ------------------------------------------- MMA issuer (even CTA)
@@ -569,6 +598,30 @@ ns_gemm_kernel(const __grid_constant__ NsParams P) {
             tc_commit_pair_multicast(&drain_bar, 0x1);
             if (!mbar_wait_cluster_bounded(&drain_bar, 0, budget, nullptr)) raise_timeout(P, abort_flag, kSiteDrain);
         }
+    } else if (kPersistent && warp == 2 + kEpiWarps) {
+        // ---------------------------------------------------------- signals
+        // Every epilogue warp reports its finished part of a tile on sig_bar;
+        // this thread adds the CTA's signals to the matrix's counter.  The
+        // release at GPU scope takes 1.6 - 2.4K cycles, a sixth of the epilogue
+        // warps' time per tile on GPT-2 Small, whose tile rate they bound.
+        if (lane == 0) {
+            int si = 0;
+            for (int seq = 0;; ++seq) {
+                const Job job = next_job(seq);
+                if (job.state == kJobTimeout) {
+                    raise_timeout(P, abort_flag, kSiteItem + 48, -2, seq);
+                    break;
+                }
+                if (job.state == kJobEnd) break;
+                if (job.stage + 1 >= ns_num_stages(P, P.cls[job.w.cls])) continue;
+                if (!mbar_wait_bounded(&sig_bar[si % kSigSlots], (si / kSigSlots) & 1, budget, abort_flag)) {
+                    raise_timeout(P, abort_flag, kSiteSignal, job.local, seq);
+                    break;
+                }
+                ++si;
+                red_release_gpu_add(P.done + job.stage * P.nmat + job.g, kEpiWarps);
+            }
+        }
     } else {
         // -------------------------------------------------------- epilogue
         uint8_t* stage_out = smem + kStages * kStageBytes;   // 1024-byte aligned
@@ -579,6 +632,7 @@ ns_gemm_kernel(const __grid_constant__ NsParams P) {
         const uint32_t tempty_leader0 = mapa_shared(smem_u32(&tempty_bar[0]), 0);
         const uint32_t tempty_leader1 = mapa_shared(smem_u32(&tempty_bar[1]), 0);
         int gi = 0;                               // product tiles so far (accumulator)
+        int si = 0;                               // reported tiles so far
         for (int seq = 0;; ++seq) {
             Job job;
             if (kPersistent) {
@@ -594,6 +648,7 @@ ns_gemm_kernel(const __grid_constant__ NsParams P) {
                 e.code = __shfl_sync(0xffffffffu, e.code, 0);
                 e.g = __shfl_sync(0xffffffffu, e.g, 0);
                 e.local = __shfl_sync(0xffffffffu, e.local, 0);
+                e.target = __shfl_sync(0xffffffffu, e.target, 0);
                 if (!ok) {
                     job.state = kJobTimeout;
                 } else {
@@ -666,7 +721,17 @@ ns_gemm_kernel(const __grid_constant__ NsParams P) {
             const int row0 = w.mt * kTileM + rank * kBM + quarter * 32;   // warp's first row
             // The first chunk's A values (and the scalars above) are in flight
             // while the accumulator is still being computed.
-            if (need_ein && nch > 0) load_ein(0, xin);
+            if (need_ein) {
+                if (kPersistent) {
+                    int ok = 1;
+                    if (lane == 0) ok = stage_done(job.stage, job.g, job.target) ? 1 : 0;
+                    if (!__shfl_sync(0xffffffffu, ok, 0)) {
+                        if (lane == 0) raise_timeout(P, abort_flag, kSiteDepLoad + 32, item, seq);
+                        break;
+                    }
+                }
+                if (nch > 0) load_ein(0, xin);
+            }
             // The epilogue warps poll with a short sleep: sixteen warps spinning
             // on this barrier cost issue slots and power the MMA and load
             // warps need (measured 0.5-1 % on every product).
@@ -797,12 +862,16 @@ ns_gemm_kernel(const __grid_constant__ NsParams P) {
                     dst[1] = sum_d;
                 }
             }
-            if (kPersistent && job.stage + 1 < ns_num_stages(P, C) && lane == 0) {
-                // This warp's part of the tile is in global memory: signal it
-                // (the last stage has no reader inside the launch).
-                bulk_wait_group_all();
-                fence_proxy_async_global();
-                red_release_gpu_add(P.done + job.stage * P.nmat + g, 1u);
+            if (kPersistent && job.stage + 1 < ns_num_stages(P, C)) {
+                // This warp's part of the tile is in global memory: report it
+                // to the signal warp (the last stage has no reader inside the
+                // launch).
+                if (lane == 0) {
+                    bulk_wait_group_all();
+                    fence_proxy_async_global();
+                    mbar_arrive(&sig_bar[si % kSigSlots]);
+                }
+                ++si;
             }
         }
         if (lane == 0) bulk_wait_group_all();     // every output store has landed
@@ -851,11 +920,12 @@ cudaError_t configure_current_device(int* pairs) {
     if (g_pairs[dev] == 0) {
         e = set_all_smem_attrs();
         if (e != cudaSuccess) return e;
-        // All instantiations have the same block shape and shared memory.
+        // One CTA per SM either way (shared memory); the persistent
+        // instantiation has the larger block.
         int n = 0;
         cudaLaunchConfig_t cfg = {};
         cfg.gridDim = dim3(2, 1, 1);
-        cfg.blockDim = dim3(kThreads, 1, 1);
+        cfg.blockDim = dim3(ns_threads(kNsPersistent), 1, 1);
         cfg.dynamicSmemBytes = kSmemBytes;
         if (cudaOccupancyMaxActiveClusters(&n, ns_gemm_kernel<kNsPersistent>, &cfg) != cudaSuccess ||
             n <= 0) {
@@ -895,7 +965,7 @@ cudaError_t launch_ns_gemm(const NsParams& P, int mode, int grid_pairs, cudaStre
     if (ce != cudaSuccess) return ce;
     const cudaError_t e = launch_chained(mode == kNsPersistent ? ns_gemm_kernel<kNsPersistent>
                                                                : ns_gemm_kernel<kNsPhased>,
-                                         2 * grid_pairs, kThreads, kSmemBytes, s, P);
+                                         2 * grid_pairs, ns_threads(mode), kSmemBytes, s, P);
     if (e != cudaSuccess) {
         cudaFuncAttributes fa{};
         if (mode == kNsPersistent)
@@ -906,7 +976,7 @@ cudaError_t launch_ns_gemm(const NsParams& P, int mode, int grid_pairs, cudaStre
                      "malt: ns_gemm_kernel<%d> launch (%d CTAs x %d threads, %zu B dynamic smem, "
                      "%zu B parameters) refused: %s; kernel uses %d registers, %zu B static "
                      "smem, allows %d threads and %d B dynamic smem per block\n",
-                     mode, 2 * grid_pairs, kThreads, kSmemBytes, sizeof(NsParams),
+                     mode, 2 * grid_pairs, ns_threads(mode), kSmemBytes, sizeof(NsParams),
                      cudaGetErrorString(e), fa.numRegs, fa.sharedSizeBytes,
                      fa.maxThreadsPerBlock, fa.maxDynamicSharedSizeBytes);
         cudaGetLastError();

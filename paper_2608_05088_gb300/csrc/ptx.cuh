@@ -82,6 +82,10 @@ __device__ __forceinline__ void cluster_sync() {
                  ::: "memory");
 }
 
+__device__ __forceinline__ void mbar_arrive(uint64_t* bar) {
+    asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_u32(bar)) : "memory");
+}
+
 // Arrive (release at CTA scope, the instruction's default) on an mbarrier of any
 // CTA of the cluster.  For signals that hand over no memory contents (an
 // accumulator that has been read): a release at cluster scope would hold the
@@ -169,7 +173,7 @@ __device__ __forceinline__ bool counter_wait_bounded(const uint32_t* ctr, uint32
     if (ld_acquire_gpu(ctr) >= target) return true;
     const uint64_t t0 = globaltimer_ns();
     for (uint32_t it = 1;; ++it) {
-        __nanosleep(64);
+        __nanosleep(20);
         if (ld_acquire_gpu(ctr) >= target) return true;
         if ((it & 15u) == 0u) {
             if (abort_flag != nullptr && *abort_flag) return false;
