@@ -189,15 +189,14 @@ __device__ __forceinline__ uint32_t pack2(float lo, float hi) {
     return u;
 }
 
-// v <- sc v + beta x + alpha on the diagonal, x 16 words of two 16-bit values.
+// v <- sc v + beta x, x 16 words of two 16-bit values.
 template <bool kF16>
-__device__ __forceinline__ void add_ein(float (&v)[32], const uint32_t* x, float sc, float beta, float alpha,
-                                        int col0, int row) {
+__device__ __forceinline__ void add_ein(float (&v)[32], const uint32_t* x, float sc, float beta) {
 #pragma unroll
     for (int j = 0; j < 32; j += 2) {
         const float2 e = unpack2<kF16>(x[j >> 1]);
-        v[j] = fmaf(beta, e.x, sc * v[j]) + (col0 + j == row ? alpha : 0.f);
-        v[j + 1] = fmaf(beta, e.y, sc * v[j + 1]) + (col0 + j + 1 == row ? alpha : 0.f);
+        v[j] = fmaf(beta, e.x, sc * v[j]);
+        v[j + 1] = fmaf(beta, e.y, sc * v[j + 1]);
     }
 }
 
@@ -719,6 +718,16 @@ ns_gemm_kernel(const __grid_constant__ NsParams P) {
             uint4 xin[4];
             uint32_t rv[32];
             const int row0 = w.mt * kTileM + rank * kBM + quarter * 32;   // warp's first row
+            // The back-map scalings of this warp's columns (lane j of chunk ch holds
+            // column 32 ch + j; 0 past N).
+            float vl[kEpiChunks];
+            if (last_bx) {
+#pragma unroll
+                for (int ch = 0; ch < kEpiChunks; ++ch) {
+                    const int col = col_base + ch * 32 + lane;
+                    vl[ch] = col < N ? (kPersistent ? __ldcg(vvec + col) : vvec[col]) : 0.f;
+                }
+            }
             // The first chunk's A values (and the scalars above) are in flight
             // while the accumulator is still being computed.
             if (need_ein) {
@@ -761,9 +770,15 @@ ns_gemm_kernel(const __grid_constant__ NsParams P) {
                 if (need_ein) {
                     const uint32_t* xw = reinterpret_cast<const uint32_t*>(xcur);
                     if (in16)
-                        add_ein<true>(v, xw, sc, op.beta, op.alpha, col0, row);
+                        add_ein<true>(v, xw, sc, op.beta);
                     else
-                        add_ein<false>(v, xw, sc, op.beta, op.alpha, col0, row);
+                        add_ein<false>(v, xw, sc, op.beta);
+                    // Rows and columns of a chunk start at multiples of 32, so
+                    // only a chunk on the diagonal holds any of it, in lane = j.
+                    if (row0 == col0) {
+#pragma unroll
+                        for (int j = 0; j < 32; ++j) v[j] += lane == j ? op.alpha : 0.f;
+                    }
                 } else {
 #pragma unroll
                     for (int j = 0; j < 32; ++j) v[j] *= sc;
@@ -826,17 +841,16 @@ ns_gemm_kernel(const __grid_constant__ NsParams P) {
                 if (last_bx) {
                     // Partial sums of O^2 and (O v)^2 over the stored (bf16) O of this
                     // row; D^2 = u_row^2 (O v)^2 is formed once per tile.  Lane j holds
-                    // v[col0 + j] and broadcasts it (columns past N contribute 0).
-                    const float vl = (col0 + lane < N)
-                                         ? (kPersistent ? __ldcg(vvec + col0 + lane) : vvec[col0 + lane])
-                                         : 0.f;
+                    // v[col0 + j] and broadcasts it.  Columns past N (ragged frames
+                    // only) hold what their accumulators held and do not count.
+                    const bool full = col0 + 32 <= N;
 #pragma unroll
                     for (int j = 0; j < 32; ++j) {
-                        const float vj = __shfl_sync(0xffffffffu, vl, j);
+                        const float vj = __shfl_sync(0xffffffffu, vl[ch], j);
                         const float2 o2 = unpack2<false>(wv[j >> 1]);
                         const float o = j & 1 ? o2.y : o2.x;
                         const float ov = o * vj;
-                        sum_o = fmaf(o, (col0 + j < N) ? o : 0.f, sum_o);
+                        sum_o = fmaf(o, full || col0 + j < N ? o : 0.f, sum_o);
                         sum_d = fmaf(ov, ov, sum_d);
                     }
                 }
