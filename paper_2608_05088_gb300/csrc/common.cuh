@@ -21,12 +21,13 @@ constexpr int kPreCols = 256;
 // Apply kernel: contiguous elements per block (O is stored in W's layout, so
 // wide and tall matrices stream alike).
 constexpr int kApplyElems = 16384;
-// Newton-Schulz GEMM: a CTA pair computes a kTileM x kBN output tile; each CTA
-// owns kBM rows of it, loads kBM rows of A and kBN/2 rows (N) of B per kBK
-// reduction slice (one 128-byte swizzle row of bf16).
+// Newton-Schulz GEMM: a CTA pair computes a kTileM x n output tile, n the set's
+// tile width; each CTA owns kBM rows of it, loads kBM rows of A and n/2 rows (N)
+// of B per kBK reduction slice (one 128-byte swizzle row of 16-bit elements).
 constexpr int kBM = 128;
 constexpr int kTileM = 2 * kBM;
-constexpr int kBN = 256;
+constexpr int kWideN = 256;
+constexpr int kNarrowN = 128;
 constexpr int kBK = 64;
 constexpr int kStages = 6;
 constexpr int kBMN = 64;            // MN extent of one 128-byte swizzle atom (bf16)
@@ -162,12 +163,14 @@ __host__ __device__ __forceinline__ int32_t entry_b(const NsEntry& e) {
 // One shape class (every matrix whose NS frame is p x q, stored batched) with
 // the tensor maps of all its buffers.
 struct NsClass {  // 64-byte aligned through its CUtensorMap members
-    CUtensorMap tmK[6];           // p x p buffers 0 .. 3 and the iterates X as K-major rows (box kBK x kBM)
+    CUtensorMap tmK[6];           // p x p buffers 0 .. 3 and the iterates X as K-major rows (box kBK x tile_n / 2)
     CUtensorMap tmXmn[2];         // the iterates as an MN-major [K][N] operand (box kBMN x kBK)
     CUtensorMap stK[6], stO;      // epilogue stores of the same buffers and of O: box 32 x 32, 64-byte swizzle
     CUtensorMap stOt;             // the O buffer as [q][p]: a tall W's O, stored in W's layout
     int32_t p, q, batch;
-    int32_t tiles_p, tiles_q;     // 256-wide tiles along p and along q
+    int32_t tile_n;               // width of an output tile
+    int32_t tiles_p, tiles_q;     // kTileM-high tiles along p, tile_n-wide ones along q
+    int32_t sym_tiles;            // tiles of one matrix in a symmetric product
     int32_t item_begin;           // first item of this class in a phased launch
     int32_t can_group;            // the shape takes the grouped form when the run may
     int32_t grouped;              // this run's form
@@ -213,7 +216,7 @@ __host__ __device__ __forceinline__ NsOp ns_op(const NsParams& P, const NsClass&
     return ns_iterated_op(iter, s - 3 * iter, iter == P.ns_steps - 1, P.a, P.b, P.c);
 }
 
-// One decoded work item: a 256 x 256 output tile of one product.
+// One decoded work item: an output tile of one product.
 struct NsWork {
     NsOp op;
     int32_t cls, b;               // class and batch slot (matrix = cls.mat_of[b])
@@ -221,10 +224,18 @@ struct NsWork {
     int32_t local;                // tile index within the matrix's product
 };
 
-// Tiles of one matrix in a product of this kind: all of them for B X, the
-// upper triangle (nt >= mt) for the symmetric Gram and polynomial products.
+// Tiles of one matrix in a product of this kind: all of them for B X, those that
+// reach the diagonal or lie above it for the symmetric Gram and p x p products.
+// Row r of tiles has those from column r * kTileM on.
+// (tile_n is the class's, a constant of the kernel)
+__host__ __device__ __forceinline__ int32_t ns_sym_row_tiles(int32_t p, int32_t tile_n, int32_t r) {
+    return (p + tile_n - 1) / tile_n - r * (kTileM / tile_n);
+}
 __host__ __device__ __forceinline__ int32_t ns_phase_tiles(const NsClass& C, int32_t kind) {
-    return kind == kBX ? C.tiles_p * C.tiles_q : C.tiles_p * (C.tiles_p + 1) / 2;
+    if (kind == kBX) return C.tiles_p * C.tiles_q;
+    int32_t n = 0;
+    for (int32_t r = 0; r < C.tiles_p; ++r) n += ns_sym_row_tiles(C.p, C.tile_n, r);
+    return n;
 }
 
 // B*X tile order.  Row by row, the tiles that run at once read every column
@@ -238,8 +249,8 @@ constexpr int64_t kBxColBytes = 32ll << 20;
 // Tile row / column of the rem-th tile of one matrix's product of this kind:
 // B*X row by row or column by column (bx_col_major), the upper triangle of
 // the symmetric products row by row.
-__host__ __device__ __forceinline__ void ns_tile_coords(const NsClass& C, int32_t kind, int32_t rem,
-                                                        int32_t* mt, int32_t* nt) {
+__host__ __device__ __forceinline__ void ns_tile_coords(const NsClass& C, int32_t tile_n, int32_t kind,
+                                                        int32_t rem, int32_t* mt, int32_t* nt) {
     if (kind == kBX) {
         if (C.bx_col_major) {
             *nt = rem / C.tiles_p;
@@ -250,13 +261,15 @@ __host__ __device__ __forceinline__ void ns_tile_coords(const NsClass& C, int32_
         }
         return;
     }
-    int32_t r = 0, u = rem;
-    while (u >= C.tiles_p - r) {
-        u -= C.tiles_p - r;
+    const int32_t step = kTileM / tile_n;
+    int32_t r = 0, u = rem, row = ns_sym_row_tiles(C.p, tile_n, 0);
+    while (u >= row) {
+        u -= row;
+        row -= step;
         ++r;
     }
     *mt = r;
-    *nt = r + u;
+    *nt = r * step + u;
 }
 
 // Blocks of the apply pass of one matrix: kApplyElems contiguous elements
@@ -266,19 +279,19 @@ __host__ __device__ __forceinline__ int32_t mat_apply_blocks(const MatDesc& d) {
 }
 
 // Item `item` of a phased launch (stage P.stage of every class that has it).
-__host__ __device__ __forceinline__ NsWork ns_decode(const NsParams& P, int32_t item) {
+__host__ __device__ __forceinline__ NsWork ns_decode(const NsParams& P, int32_t tile_n, int32_t item) {
     NsWork w;
     int32_t c = 0;
     while (c + 1 < P.nclasses && item >= P.cls[c + 1].item_begin) ++c;
     const NsClass& C = P.cls[c];
     w.op = ns_op(P, C, P.stage);
     const int32_t local = item - C.item_begin;
-    const int32_t per = ns_phase_tiles(C, w.op.kind);
+    const int32_t per = w.op.kind == kBX ? C.tiles_p * C.tiles_q : C.sym_tiles;
     w.cls = c;
     w.b = local / per;
     const int32_t rem = local - w.b * per;
     w.local = rem;
-    ns_tile_coords(C, w.op.kind, rem, &w.mt, &w.nt);
+    ns_tile_coords(C, tile_n, w.op.kind, rem, &w.mt, &w.nt);
     return w;
 }
 

@@ -88,7 +88,8 @@ struct ShapeClass {
     __nv_bfloat16* P[4] = {nullptr, nullptr, nullptr, nullptr};
     __nv_bfloat16* O = nullptr;                  // last iterate, per matrix in W's layout:
                                                  // [p][q] (wide) or [q][p] (tall)
-    CUtensorMap tmK[6] = {}, tmXmn[2];          // 128-row K-major boxes; 64x64 MN boxes
+    int tile_n = kWideN;                         // width of the set's output tiles
+    CUtensorMap tmK[6] = {}, tmXmn[2];           // K-major boxes of tile_n / 2 rows; 64 x 64 MN boxes
     CUtensorMap stK[6] = {}, stO, stOt;         // epilogue store maps (stOt: O as [q][p])
 };
 
@@ -312,7 +313,17 @@ constexpr int kStatusWords = 8;
 
 // Per-matrix descriptions and shape classes (one per NS frame p x q, in order
 // of first appearance).  Host only.
-void build_classes(const malt_param_t* params, int n, std::vector<MatDesc>& hmats,
+//
+// Tile width: 256 columns, or 128 for a set of few tiles (counted 256 wide, per
+// product).  There CTA pairs idle and a product takes its latency; half as wide, a
+// tile's MMAs and its epilogue (2.3 us of a product's 7.8) take half the time.
+// Newton-Schulz at k = 5, us per step, wide / narrow: one 256 x 512 matrix 118 / 85,
+// one 1280 x 1280 196 / 158, 16 of 256 x 2048 (16 symmetric and 128 B*X tiles)
+// 161 / 132, 8 of 768 x 768 (48 and 72) 172 / 144, one 2048 x 2048 (36 and 64)
+// 259 / 263, 8 of 1024 x 1024 (80 and 128) 205 / 244.  The wide tile loads a quarter
+// less per flop.  narrow_tiles false: 256 always (malt_ns_schedule's tables).
+constexpr int kNarrowMaxSym = 48, kNarrowMaxBx = 128;
+void build_classes(const malt_param_t* params, int n, bool narrow_tiles, std::vector<MatDesc>& hmats,
                    std::vector<ShapeClass>& classes) {
     hmats.resize(n);
     std::map<std::pair<int, int>, int> cls_of;
@@ -348,14 +359,23 @@ void build_classes(const malt_param_t* params, int n, std::vector<MatDesc>& hmat
         d.stat_cb = (c + kStatCols - 1) / kStatCols;
         d.pre_tr = (m + kPreRows - 1) / kPreRows;
         d.pre_tc = (c + kPreCols - 1) / kPreCols;
-        d.ns_tiles = ((p + kTileM - 1) / kTileM) * ((q + kBN - 1) / kBN);
     }
     int64_t tiles = 0;                 // of one symmetric product over the set
     for (const ShapeClass& C : classes) {
         const int64_t tp = (C.p + kTileM - 1) / kTileM;
         tiles += tp * (tp + 1) / 2 * C.batch;
     }
-    for (ShapeClass& C : classes) C.can_group = ns_grouped_shape(C.p, C.q, tiles);
+    int64_t bx_tiles = 0;              // of B*X
+    for (const ShapeClass& C : classes)
+        bx_tiles += static_cast<int64_t>((C.p + kTileM - 1) / kTileM) * ((C.q + kWideN - 1) / kWideN) * C.batch;
+    for (ShapeClass& C : classes) {
+        C.can_group = ns_grouped_shape(C.p, C.q, tiles);
+        C.tile_n = narrow_tiles && tiles <= kNarrowMaxSym && bx_tiles <= kNarrowMaxBx ? kNarrowN : kWideN;
+    }
+    for (MatDesc& d : hmats) {
+        const int tile_n = classes[d.cls].tile_n;
+        d.ns_tiles = ((d.p + kTileM - 1) / kTileM) * ((d.q + tile_n - 1) / tile_n);
+    }
 }
 
 // Newton-Schulz work lists: classes ordered by Gram reduction length (q, then
@@ -396,7 +416,9 @@ void plan_ns_groups(const std::vector<ShapeClass>& classes, int nmat, std::vecto
             C.q = S.q;
             C.batch = S.batch;
             C.tiles_p = (S.p + kTileM - 1) / kTileM;
-            C.tiles_q = (S.q + kBN - 1) / kBN;
+            C.tile_n = S.tile_n;
+            C.tiles_q = (S.q + S.tile_n - 1) / S.tile_n;
+            C.sym_tiles = ns_phase_tiles(C, kGram);
             C.bx_col_major = static_cast<int64_t>(S.p) * S.q * 2 > kBxColBytes ? 1 : 0;
             C.mat_of = S.d_mat_of;
             C.A = reinterpret_cast<const uint16_t*>(S.P[0]);
@@ -472,7 +494,7 @@ int plan_and_allocate(malt_state* st, const malt_param_t* params, int n) {
     st->nmat = n;
     st->shape0.assign(params, params + n);
     st->wcopy.assign(n, nullptr);
-    build_classes(params, n, st->hmats, st->classes);
+    build_classes(params, n, true, st->hmats, st->classes);
 
     // Workspace layout.
     Carver cv;
@@ -649,12 +671,12 @@ int plan_and_allocate(malt_state* st, const malt_param_t* params, int n) {
         // (a map moves 16-bit elements; whether they are bf16 or fp16 is the
         // operation's business)
         for (int b = 0; b < 2; ++b) {
-            ok &= encode_3d(&C.tmK[kBufX + b], C.X[b], C.q, C.p, C.batch, kBM);
+            ok &= encode_3d(&C.tmK[kBufX + b], C.X[b], C.q, C.p, C.batch, C.tile_n / 2);
             ok &= encode_3d(&C.tmXmn[b], C.X[b], C.q, C.p, C.batch, kBK);
             ok &= encode_store(&C.stK[kBufX + b], C.X[b], C.q, C.p, C.batch);
         }
         for (int b = 0; b < (C.can_group ? 4 : 2); ++b) {
-            ok &= encode_3d(&C.tmK[b], C.P[b], C.p, C.p, C.batch, kBM);
+            ok &= encode_3d(&C.tmK[b], C.P[b], C.p, C.p, C.batch, C.tile_n / 2);
             ok &= encode_store(&C.stK[b], C.P[b], C.p, C.p, C.batch);
         }
         ok &= encode_store(&C.stO, C.O, C.q, C.p, C.batch);
@@ -1292,7 +1314,7 @@ int malt_ns_schedule(const malt_param_t* params, int32_t n, int32_t ns_steps, in
             return MALT_ERR_UNSUPPORTED;
     std::vector<MatDesc> hmats;
     std::vector<ShapeClass> classes;
-    build_classes(params, n, hmats, classes);
+    build_classes(params, n, false, hmats, classes);
     std::vector<NsParams> groups;
     std::vector<std::vector<int>> slot_class;
     plan_ns_groups(classes, n, groups, &slot_class);
@@ -1335,7 +1357,7 @@ int malt_ns_plan(int64_t rows, int64_t cols, int32_t n, const malt_hparams_t* hp
     std::vector<MatDesc> hmats;
     std::vector<ShapeClass> classes;
     const std::vector<malt_param_t> set(static_cast<size_t>(n), p);
-    build_classes(set.data(), n, hmats, classes);
+    build_classes(set.data(), n, true, hmats, classes);
     std::vector<NsParams> groups;
     plan_ns_groups(classes, n, groups);
     NsParams& G = groups[0];

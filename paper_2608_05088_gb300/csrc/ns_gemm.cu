@@ -29,7 +29,7 @@
 // of a symmetric tile), so the apply pass streams every matrix the same way.
 //
 // Work split.  A cluster of two CTAs (a CTA pair on two SMs) computes one
-// 256 x 256 output tile per turn: CTA r owns rows [128 r, 128 r + 128) of the
+// 256 x 256 output tile per turn (256 x 128 in sets of few tiles, build_classes): CTA r owns rows [128 r, 128 r + 128) of the
 // tile in its own TMEM.  Per 64-wide reduction slice each CTA loads its 128
 // rows of A and its half (128 N-rows or N-columns) of B, 32 KB, into one of
 // kStages slice slots; the MMA, issued by one thread of the even CTA, reads
@@ -95,25 +95,33 @@ namespace {
 constexpr int kEpiWarps = kEpiWarpsPerCta;
 // A persistent launch has one more warp, which signals finished tiles.
 constexpr int ns_threads(int mode) { return 64 + 32 * kEpiWarps + (mode == kNsPersistent ? 32 : 0); }
-constexpr int kEpiCols = kBN / (kEpiWarps / 4);        // accumulator columns per warp
-constexpr int kEpiChunks = kEpiCols / 32;
-constexpr int kHalfN = kBN / 2;                        // B rows (or columns) per CTA
 constexpr uint32_t kABytes = kBM * kBK * 2;            // 16 KB
-constexpr uint32_t kBBytes = kHalfN * kBK * 2;         // 16 KB
-constexpr uint32_t kStageBytes = kABytes + kBBytes;     // one 64-wide reduction slice
+constexpr uint32_t kMnBoxBytes = kBMN * kBK * 2;       // one 64 x 64 MN-major box
+constexpr uint32_t kMnLbo = kMnBoxBytes;               // next 64 MN-elements
+
+// What follows from the width kN of an output tile.
+template <int kN>
+struct Tile {
+    static constexpr int kEpiCols = kN / (kEpiWarps / 4);   // accumulator columns per warp
+    static constexpr int kEpiChunks = kEpiCols / 32;
+    static constexpr int kHalfN = kN / 2;                   // B rows (or columns) per CTA
+    static constexpr uint32_t kBBytes = kHalfN * kBK * 2;   // 16 KB (wide), 8 KB (narrow)
+    static constexpr uint32_t kStageBytes = kABytes + kBBytes;   // one 64-wide reduction slice
+    static constexpr uint32_t kTmemCols = 2 * kN;
+    static_assert(kTmemCols <= 512, "two accumulators must fit in TMEM");
+    static_assert(kHalfN % kBMN == 0, "B half must be whole MN-major boxes");
+    static_assert(kTileM % kN == 0, "a row of tiles starts on the diagonal");
+};
 // Ring granularity: the producer fills, and the MMA thread waits for and
 // releases, kGroup slices at a time.  A barrier wait and a commit sit on the
 // MMA issue path once per kGroup slices (8 MMAs) instead of once per 4 MMAs.
 constexpr int kGroup = 2;
 constexpr int kRing = kStages / kGroup;
 static_assert(kStages % kGroup == 0, "the slice slots form whole ring stages");
-constexpr uint32_t kTmemCols = 2 * kBN;
-constexpr uint32_t kMnBoxBytes = kBMN * kBK * 2;       // one 64 x 64 MN-major box
-constexpr uint32_t kMnLbo = kMnBoxBytes;               // next 64 MN-elements
 constexpr uint32_t kStoreBoxBytes = 32 * 32 * 2;      // one 32 x 32 bf16 output box
 constexpr uint32_t kStageOutBytes = 2 * kStoreBoxBytes * kEpiWarps;  // double-buffered per warp
 constexpr size_t kSmemBytes =
-    static_cast<size_t>(kStages) * kStageBytes + kStageOutBytes + 1024;
+    static_cast<size_t>(kStages) * Tile<kWideN>::kStageBytes + kStageOutBytes + 1024;
 constexpr uint16_t kPairMask = 0x3;
 // Persistent schedule: slots of the item ring (how far the scheduler may run
 // ahead of the slowest reader, the epilogue), and the readers of each slot:
@@ -129,10 +137,7 @@ static_assert(2 * kEpiWarps == static_cast<int>(kNsSignalsPerTile),
 constexpr int kSigSlots = 4;
 
 static_assert(kBK * 2 == 128, "one K slice must be one 128-byte swizzle row");
-static_assert(kTmemCols <= 512, "two accumulators must fit in TMEM");
-static_assert(kHalfN % kBMN == 0, "B half must be whole MN-major boxes");
 static_assert(kEpiWarps == 8, "epilogue layout assumes two warps per lane quarter");
-static_assert(kTileM == kBN, "symmetric products need square tiles");
 
 // Operands and output of one work item.
 struct Ops {
@@ -154,11 +159,13 @@ __device__ __forceinline__ Ops item_operands(const NsParams& P, const NsWork& w)
 // Bytes CTA `rank` loads for one reduction slice of a tile.  Boxes that lie
 // wholly past M or N are skipped: they only feed accumulator rows / columns
 // that are never stored.
+template <int kN>
 __device__ __forceinline__ uint32_t slice_bytes(const Ops& op, const NsWork& w, int rank,
                                                 bool b_mn, int* nbox_b) {
     uint32_t bytes = 0;
     if (w.mt * kTileM + rank * kBM < op.M) bytes += kABytes;
-    const int n0 = w.nt * kBN + rank * kHalfN;
+    constexpr int kHalfN = Tile<kN>::kHalfN;
+    const int n0 = w.nt * kN + rank * kHalfN;
     int nb = 0;
     if (b_mn) {
         for (int j = 0; j < kHalfN / kBMN; ++j)
@@ -166,7 +173,7 @@ __device__ __forceinline__ uint32_t slice_bytes(const Ops& op, const NsWork& w, 
         bytes += nb * kMnBoxBytes;
     } else if (n0 < op.N) {
         nb = 1;
-        bytes += kBBytes;
+        bytes += Tile<kN>::kBBytes;
     }
     *nbox_b = nb;
     return bytes;
@@ -242,6 +249,7 @@ struct Job {
     NsWork w;
 };
 
+template <int kN>
 __device__ __forceinline__ Job job_of_entry(const NsParams& P, const NsEntry& e) {
     Job j;
     if (e.g < 0) {
@@ -257,16 +265,18 @@ __device__ __forceinline__ Job job_of_entry(const NsParams& P, const NsEntry& e)
     j.w.op = ns_op(P, P.cls[j.w.cls], j.stage);
     j.w.b = entry_b(e);
     j.w.local = e.local;
-    ns_tile_coords(P.cls[j.w.cls], j.w.op.kind, e.local, &j.w.mt, &j.w.nt);
+    ns_tile_coords(P.cls[j.w.cls], kN, j.w.op.kind, e.local, &j.w.mt, &j.w.nt);
     return j;
 }
 
 }  // namespace
 
-template <int kMode>
+template <int kMode, int kN>
 __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(ns_threads(kMode), 1)
 ns_gemm_kernel(const __grid_constant__ NsParams P) {
     constexpr bool kPersistent = kMode == kNsPersistent;   // table-driven, claimed dynamically
+    constexpr int kHalfN = Tile<kN>::kHalfN, kEpiCols = Tile<kN>::kEpiCols, kEpiChunks = Tile<kN>::kEpiChunks;
+    constexpr uint32_t kStageBytes = Tile<kN>::kStageBytes, kTmemCols = Tile<kN>::kTmemCols;
     extern __shared__ uint8_t smem_raw[];
     __shared__ __align__(8) uint64_t full_bar[kRing];
     __shared__ __align__(8) uint64_t empty_bar[kRing];
@@ -350,7 +360,7 @@ ns_gemm_kernel(const __grid_constant__ NsParams P) {
             return j;
         }
         j.state = kJobWork;
-        j.w = ns_decode(P, static_cast<int>(it));
+        j.w = ns_decode(P, kN, static_cast<int>(it));
         j.stage = P.stage;
         j.g = -1;
         j.local = j.w.local;
@@ -382,7 +392,7 @@ ns_gemm_kernel(const __grid_constant__ NsParams P) {
             j.state = kJobTimeout;
             return j;
         }
-        return job_of_entry(P, e);
+        return job_of_entry<kN>(P, e);
     };
     auto next_job = [&](int seq) -> Job { return kPersistent ? ring_job(seq) : static_job(seq); };
     // Scheduler (odd CTA): the table entry of the next claimed item (an end
@@ -460,11 +470,11 @@ ns_gemm_kernel(const __grid_constant__ NsParams P) {
                 // A diagonal tile of a product of a matrix with itself: each CTA's
                 // half of B is its own rows of A, so B is not loaded and the MMA
                 // reads A twice.
-                const bool same_ab = w.op.a == w.op.b && w.mt == w.nt;
+                const bool same_ab = kN == kTileM && w.op.a == w.op.b && w.mt == w.nt;
                 const int nkb = (op.K + kBK - 1) / kBK;
                 int nb_self = 0, nb_peer = 0;
-                uint32_t bytes_pair = slice_bytes(op, w, rank, b_mn, &nb_self) +
-                                      slice_bytes(op, w, rank ^ 1, b_mn, &nb_peer);
+                uint32_t bytes_pair = slice_bytes<kN>(op, w, rank, b_mn, &nb_self) +
+                                      slice_bytes<kN>(op, w, rank ^ 1, b_mn, &nb_peer);
                 if (same_ab) {
                     nb_self = 0;
                     bytes_pair = (w.mt * kTileM < op.M ? kABytes : 0u) +
@@ -472,7 +482,7 @@ ns_gemm_kernel(const __grid_constant__ NsParams P) {
                 }
                 const bool load_a = w.mt * kTileM + rank * kBM < op.M;
                 const int a_row = w.mt * kTileM + rank * kBM;
-                const int n0 = w.nt * kBN + rank * kHalfN;
+                const int n0 = w.nt * kN + rank * kHalfN;
                 bool ok = true;
                 for (int k0 = 0; k0 < nkb; k0 += kGroup) {
                     if (!mbar_wait_cluster_bounded(&empty_bar[stage], phase ^ 1u, budget, abort_flag)) {
@@ -486,7 +496,11 @@ ns_gemm_kernel(const __grid_constant__ NsParams P) {
                     for (int j = 0; j < nsub; ++j) {
                         const int kb = k0 + j;
                         uint8_t* sa = smem + (stage * kGroup + j) * kStageBytes;
-                        if (load_a) tma_load_3d_pair(sa, op.a, kb * kBK, a_row, w.b, fb);
+                        if (load_a) {
+#pragma unroll
+                            for (int h = 0; h < kBM; h += kHalfN)
+                                tma_load_3d_pair(sa + h * (kBK * 2), op.a, kb * kBK, a_row + h, w.b, fb);
+                        }
                         if (b_mn) {
                             for (int jb = 0; jb < nb_self; ++jb)
                                 tma_load_3d_pair(sa + kABytes + jb * kMnBoxBytes, op.b,
@@ -541,12 +555,12 @@ ns_gemm_kernel(const __grid_constant__ NsParams P) {
                 const int item = job.local;
                 const NsWork& w = job.w;
                 const bool b_mn = w.op.kind == kBX;
-                const bool same_ab = w.op.a == w.op.b && w.mt == w.nt;
+                const bool same_ab = kN == kTileM && w.op.a == w.op.b && w.mt == w.nt;
                 const int K = w.op.kind == kGram ? P.cls[w.cls].q : P.cls[w.cls].p;
-                const uint32_t idesc = b_mn ? (w.op.f16 ? idesc_16bit_f32(kTileM, kBN, true, true)
-                                                        : idesc_16bit_f32(kTileM, kBN, false, true))
-                                            : (w.op.f16 ? idesc_16bit_f32(kTileM, kBN, true, false)
-                                                        : idesc_16bit_f32(kTileM, kBN, false, false));
+                const uint32_t idesc = b_mn ? (w.op.f16 ? idesc_16bit_f32(kTileM, kN, true, true)
+                                                        : idesc_16bit_f32(kTileM, kN, false, true))
+                                            : (w.op.f16 ? idesc_16bit_f32(kTileM, kN, true, false)
+                                                        : idesc_16bit_f32(kTileM, kN, false, false));
                 const int nkb = (K + kBK - 1) / kBK;
                 const uint32_t acc = gi & 1, acc_phase = (gi >> 1) & 1;
                 ++gi;
@@ -555,7 +569,7 @@ ns_gemm_kernel(const __grid_constant__ NsParams P) {
                     break;
                 }
                 tc_fence_after();
-                const uint32_t d_tmem = tmem_base + acc * kBN;
+                const uint32_t d_tmem = tmem_base + acc * kN;
                 bool ok = true;
                 for (int k0 = 0; k0 < nkb; k0 += kGroup) {
                     if (!mbar_wait_cluster_bounded(&full_bar[stage], phase, budget, abort_flag)) {
@@ -651,7 +665,7 @@ ns_gemm_kernel(const __grid_constant__ NsParams P) {
                 if (!ok) {
                     job.state = kJobTimeout;
                 } else {
-                    job = job_of_entry(P, e);
+                    job = job_of_entry<kN>(P, e);
                 }
             } else {
                 job = static_job(seq);
@@ -694,10 +708,10 @@ ns_gemm_kernel(const __grid_constant__ NsParams P) {
             const float urow = (last_bx && rok) ? (kPersistent ? __ldcg(uvec + row) : uvec[row]) : 0.f;
             float sum_o = 0.f, sum_d = 0.f;
 
-            const int col_base = w.nt * kBN + colw;     // first output column of this warp
+            const int col_base = w.nt * kN + colw;     // first output column of this warp
             const int nch = max(0, min(kEpiChunks, (N - col_base + 31) / 32));
             const uint32_t tbase = tmem_base + (static_cast<uint32_t>(quarter * 32) << 16) +
-                                   acc * kBN + colw;
+                                   acc * kN + colw;
             auto load_ein = [&](int ch, uint4 (&dst)[4]) {
                 const int col0 = col_base + ch * 32;
 #pragma unroll
@@ -808,7 +822,7 @@ ns_gemm_kernel(const __grid_constant__ NsParams P) {
                     }
                     obuf ^= 1;
                 }
-                if (store_t || (sym && w.nt != w.mt)) {
+                if (store_t || (sym && w.nt * kN >= (w.mt + 1) * kTileM)) {
                     // Mirror an off-diagonal tile of the symmetric product, or
                     // store a tall matrix's O in W's layout: the transposed chunk
                     // (box row = column j, 32 rows of this warp) goes to rows
@@ -905,16 +919,22 @@ size_t ns_gemm_smem_bytes() { return kSmemBytes; }
 
 namespace {
 
-template <int kMode>
-cudaError_t set_smem_attr() {
-    return cudaFuncSetAttribute(ns_gemm_kernel<kMode>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                static_cast<int>(kSmemBytes));
+using NsKernel = void (*)(const NsParams);
+
+NsKernel ns_kernel(int mode, int tile_n) {
+    if (mode == kNsPersistent)
+        return tile_n == kNarrowN ? ns_gemm_kernel<kNsPersistent, kNarrowN> : ns_gemm_kernel<kNsPersistent, kWideN>;
+    return tile_n == kNarrowN ? ns_gemm_kernel<kNsPhased, kNarrowN> : ns_gemm_kernel<kNsPhased, kWideN>;
 }
 
 cudaError_t set_all_smem_attrs() {
-    cudaError_t e = set_smem_attr<kNsPhased>();
-    if (e == cudaSuccess) e = set_smem_attr<kNsPersistent>();
-    return e;
+    for (int mode : {kNsPhased, kNsPersistent})
+        for (int n : {kWideN, kNarrowN}) {
+            const cudaError_t e = cudaFuncSetAttribute(ns_kernel(mode, n), cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                                       static_cast<int>(kSmemBytes));
+            if (e != cudaSuccess) return e;
+        }
+    return cudaSuccess;
 }
 
 // Per-device one-time set-up: the shared-memory opt-in of every
@@ -941,7 +961,7 @@ cudaError_t configure_current_device(int* pairs) {
         cfg.gridDim = dim3(2, 1, 1);
         cfg.blockDim = dim3(ns_threads(kNsPersistent), 1, 1);
         cfg.dynamicSmemBytes = kSmemBytes;
-        if (cudaOccupancyMaxActiveClusters(&n, ns_gemm_kernel<kNsPersistent>, &cfg) != cudaSuccess ||
+        if (cudaOccupancyMaxActiveClusters(&n, ns_kernel(kNsPersistent, kWideN), &cfg) != cudaSuccess ||
             n <= 0) {
             cudaGetLastError();
             int sms = 0;
@@ -977,15 +997,11 @@ cudaError_t ns_gemm_configure() {
 cudaError_t launch_ns_gemm(const NsParams& P, int mode, int grid_pairs, cudaStream_t s) {
     const cudaError_t ce = ns_gemm_configure();
     if (ce != cudaSuccess) return ce;
-    const cudaError_t e = launch_chained(mode == kNsPersistent ? ns_gemm_kernel<kNsPersistent>
-                                                               : ns_gemm_kernel<kNsPhased>,
-                                         2 * grid_pairs, ns_threads(mode), kSmemBytes, s, P);
+    const NsKernel kernel = ns_kernel(mode, P.cls[0].tile_n);
+    const cudaError_t e = launch_chained(kernel, 2 * grid_pairs, ns_threads(mode), kSmemBytes, s, P);
     if (e != cudaSuccess) {
         cudaFuncAttributes fa{};
-        if (mode == kNsPersistent)
-            cudaFuncGetAttributes(&fa, ns_gemm_kernel<kNsPersistent>);
-        else
-            cudaFuncGetAttributes(&fa, ns_gemm_kernel<kNsPhased>);
+        cudaFuncGetAttributes(&fa, kernel);
         std::fprintf(stderr,
                      "malt: ns_gemm_kernel<%d> launch (%d CTAs x %d threads, %zu B dynamic smem, "
                      "%zu B parameters) refused: %s; kernel uses %d registers, %zu B static "
