@@ -20,6 +20,7 @@ struct BindParams {
 // registered).  The padding is zero at init and every stage keeps it zero.
 constexpr int kPadChunk = 48;      // matrices per pad / unpad launch
 constexpr int kPadRows = 8;        // rows per block (one warp per row)
+constexpr int kPadCols = 256;      // columns per block
 struct PadEntry {
     void* w_user;  void* w_pad;    // W (bf16 when w_bf16, else fp32)
     const void* g_user; void* g_pad;   // G (bf16 when g_bf16, else fp32)

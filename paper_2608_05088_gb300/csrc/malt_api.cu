@@ -784,7 +784,7 @@ int run_padding(malt_state* st, const malt_param_t* params, bool in, cudaStream_
             e.w_bf16 = p.w_dtype == MALT_BF16;
             e.g_bf16 = p.g_dtype == MALT_BF16;
             e.block_begin = blocks;
-            blocks += static_cast<int32_t>((p.rows + kPadRows - 1) / kPadRows);
+            blocks += static_cast<int32_t>((p.rows + kPadRows - 1) / kPadRows * ((p.cols + kPadCols - 1) / kPadCols));
         }
         LaunchScope ls(st, MALT_KIND_PAD, s);
         MALT_CUDA(launch_pad(P, blocks, in, s), in ? "pad_kernel (in)" : "pad_kernel (out)");

@@ -38,54 +38,70 @@ __global__ void bind_kernel(const __grid_constant__ BindParams P, UserPtrs* __re
 }
 
 // ------------------------------------------------------------ pad / unpad
-// One block copies kPadRows rows of one matrix (one warp per row, lanes along
-// the row); the matrix's first block also copies l and r.
-template <typename T>
-__device__ __forceinline__ void copy_row(const T* __restrict__ src, T* __restrict__ dst, int n,
-                                         int lane) {
-    for (int j = lane; j < n; j += 32) dst[j] = src[j];
+// A block copies kPadRows rows x kPadCols columns of one matrix, a warp per row,
+// and the blocks of the matrix's first row band also its l and r.  The rows start at
+// any element, so accesses are single elements, coalesced across the lanes; every
+// lane has kPadCols / 32 of them in flight per buffer, so that a block waits for
+// memory once (a row at a time with one in flight, the two launches of six matrices
+// of 77 to 515 rows took 42 us).
+// Row segments of W (or G) in either type: 16-bit elements in the low halves of v.
+__device__ __forceinline__ void load_any(const void* p, bool half, size_t off, int n, int lane,
+                                         uint32_t (&v)[kPadCols / 32]) {
+#pragma unroll
+    for (int k = 0; k < kPadCols / 32; ++k) {
+        const int j = lane + 32 * k;
+        if (j < n) v[k] = half ? static_cast<const uint16_t*>(p)[off + j] : static_cast<const uint32_t*>(p)[off + j];
+    }
+}
+
+__device__ __forceinline__ void store_any(void* p, bool half, size_t off, int n, int lane,
+                                          const uint32_t (&v)[kPadCols / 32]) {
+#pragma unroll
+    for (int k = 0; k < kPadCols / 32; ++k) {
+        const int j = lane + 32 * k;
+        if (j >= n) continue;
+        if (half)
+            static_cast<uint16_t*>(p)[off + j] = static_cast<uint16_t>(v[k]);
+        else
+            static_cast<uint32_t*>(p)[off + j] = v[k];
+    }
 }
 
 template <bool kIn>
-__global__ void __launch_bounds__(256) pad_kernel(const __grid_constant__ PadParams P) {
+__global__ void __launch_bounds__(32 * kPadRows) pad_kernel(const __grid_constant__ PadParams P) {
     chain_wait();
     int k = 0;
     while (k + 1 < P.count && P.e[k + 1].block_begin <= static_cast<int32_t>(blockIdx.x)) ++k;
     const PadEntry& e = P.e[k];
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int row = (static_cast<int>(blockIdx.x) - e.block_begin) * kPadRows + warp;
+    const int local = static_cast<int>(blockIdx.x) - e.block_begin;
+    const int segs = (e.n + kPadCols - 1) / kPadCols;
+    const int band = local / segs, col = (local - band * segs) * kPadCols;
+    const int row = band * kPadRows + warp;
+    const int n = min(kPadCols, e.n - col);                       // columns of this block
     if (row < e.m) {
-        const size_t u = static_cast<size_t>(row) * e.n;      // caller layout, ld = n
-        const size_t q = static_cast<size_t>(row) * e.n8;     // padded layout, ld = n8
-        if (kIn) {
-            if (e.w_bf16)
-                copy_row(static_cast<const uint16_t*>(e.w_user) + u, static_cast<uint16_t*>(e.w_pad) + q, e.n, lane);
-            else
-                copy_row(static_cast<const float*>(e.w_user) + u, static_cast<float*>(e.w_pad) + q, e.n, lane);
-            if (e.g_bf16)
-                copy_row(static_cast<const uint16_t*>(e.g_user) + u, static_cast<uint16_t*>(e.g_pad) + q, e.n, lane);
-            else
-                copy_row(static_cast<const float*>(e.g_user) + u, static_cast<float*>(e.g_pad) + q, e.n, lane);
-            copy_row<float>(e.m_user + u, e.m_pad + q, e.n, lane);
-        } else {
-            if (e.w_bf16) {
-                copy_row(static_cast<const uint16_t*>(e.w_pad) + q, static_cast<uint16_t*>(e.w_user) + u, e.n, lane);
-            } else {
-                const float* src = static_cast<const float*>(e.w_pad) + q;
-                copy_row(src, static_cast<float*>(e.w_user) + u, e.n, lane);
-                if (e.wcopy_user != nullptr) {
-                    __nv_bfloat16* c = static_cast<__nv_bfloat16*>(e.wcopy_user) + u;
-                    for (int j = lane; j < e.n; j += 32) c[j] = __float2bfloat16_rn(src[j]);
-                }
-            }
-            copy_row<float>(e.m_pad + q, e.m_user + u, e.n, lane);
+        const size_t u = static_cast<size_t>(row) * e.n + col;      // caller layout, ld = n
+        const size_t q = static_cast<size_t>(row) * e.n8 + col;     // padded layout, ld = n8
+        uint32_t w[kPadCols / 32], g[kPadCols / 32], m[kPadCols / 32];
+        load_any(kIn ? e.w_user : e.w_pad, e.w_bf16, kIn ? u : q, n, lane, w);
+        if (kIn) load_any(e.g_user, e.g_bf16, u, n, lane, g);
+        load_any(kIn ? e.m_user : e.m_pad, false, kIn ? u : q, n, lane, m);
+        store_any(kIn ? e.w_pad : e.w_user, e.w_bf16, kIn ? q : u, n, lane, w);
+        if (kIn) store_any(e.g_pad, e.g_bf16, q, n, lane, g);
+        store_any(kIn ? e.m_pad : e.m_user, false, kIn ? q : u, n, lane, m);
+        if (!kIn && !e.w_bf16 && e.wcopy_user != nullptr) {
+            __nv_bfloat16* c = static_cast<__nv_bfloat16*>(e.wcopy_user) + u;
+#pragma unroll
+            for (int i = 0; i < kPadCols / 32; ++i)
+                if (lane + 32 * i < n) c[lane + 32 * i] = __float2bfloat16_rn(__uint_as_float(w[i]));
         }
     }
-    if (static_cast<int>(blockIdx.x) == e.block_begin) {
-        for (int i = threadIdx.x; i < e.m; i += blockDim.x) {
+    if (band == 0) {
+        const int stride = segs * blockDim.x, first = (local % segs) * blockDim.x + threadIdx.x;
+        for (int i = first; i < e.m; i += stride) {
             if (kIn) e.l_pad[i] = e.l_user[i]; else e.l_user[i] = e.l_pad[i];
         }
-        for (int j = threadIdx.x; j < e.n; j += blockDim.x) {
+        for (int j = first; j < e.n; j += stride) {
             if (kIn) e.r_pad[j] = e.r_user[j]; else e.r_user[j] = e.r_pad[j];
         }
     }
@@ -229,7 +245,7 @@ cudaError_t launch_bind(const BindParams& P, UserPtrs* table, cudaStream_t s) {
 }
 
 cudaError_t launch_pad(const PadParams& P, int32_t blocks, bool in, cudaStream_t s) {
-    return launch_chained(in ? pad_kernel<true> : pad_kernel<false>, blocks, 256, 0, s, P);
+    return launch_chained(in ? pad_kernel<true> : pad_kernel<false>, blocks, 32 * kPadRows, 0, s, P);
 }
 
 cudaError_t launch_stats(const MatDesc* mats, const UserPtrs* ptrs, const int32_t* pref,
