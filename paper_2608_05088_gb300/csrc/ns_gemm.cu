@@ -131,10 +131,13 @@ constexpr int kNoItem = -0x7fffffff;   // never stored in the ring
 constexpr uint32_t kItemReaders = 5 + 2 * kEpiWarps;
 static_assert(2 * kEpiWarps == static_cast<int>(kNsSignalsPerTile),
               "a finished tile counts one signal per epilogue warp of the pair");
-// Signalled tiles whose stores the epilogue warps may still be reporting: a
-// warp reaches tile i + 4 only after every warp has released the accumulator
-// of tile i + 2, that is, has reported tile i.
+// Phases of sig_bar in flight.  A slot is used again by the tile kSigSlots
+// reported tiles later, at the earliest by the item kSigSlots later, which is
+// published only after the signal warp has seen this one's phase complete (it
+// frees the item's ring slot then) and processed only after every epilogue warp has
+// arrived on it (each releases the accumulators of the tiles between after that).
 constexpr int kSigSlots = 4;
+static_assert(kSigSlots >= kItemSlots, "a phase of sig_bar is seen before the slot is used again");
 
 static_assert(kBK * 2 == 128, "one K slice must be one 128-byte swizzle row");
 static_assert(kEpiWarps == 8, "epilogue layout assumes two warps per lane quarter");
@@ -367,8 +370,14 @@ ns_gemm_kernel(const __grid_constant__ NsParams P) {
         j.target = 0;
         return j;
     };
-    // The ring entry of sequence number seq (false when the wait gave up).
-    auto ring_entry = [&](int seq, NsEntry& e) -> bool {
+    // The ring entry of sequence number seq (false when the wait gave up); its
+    // reader then frees the slot with ring_free.
+    auto ring_free = [&](int seq) {
+        // The slot's barrier lives in the odd CTA, with the scheduler.  The arrive
+        // carries no data, so it is relaxed.
+        mbar_arrive_cluster_relaxed(mapa_shared(smem_u32(&item_empty[seq % kItemSlots]), 1));
+    };
+    auto ring_peek = [&](int seq, NsEntry& e) -> bool {
         const int slot = seq % kItemSlots;
         const uint32_t par = static_cast<uint32_t>(seq / kItemSlots) & 1u;
         if (!mbar_wait_cluster_bounded(&item_full[slot], par, budget, abort_flag)) return false;
@@ -377,12 +386,13 @@ ns_gemm_kernel(const __grid_constant__ NsParams P) {
         e.g = v[1];
         e.local = v[2];
         e.target = static_cast<uint32_t>(v[3]);
-        // Free the slot (its barrier lives in the odd CTA, with the
-        // scheduler).  The arrive carries no data, so it is relaxed; it is
-        // issued only once the slot's value is in hand (the branch depends on
+        return true;
+    };
+    auto ring_entry = [&](int seq, NsEntry& e) -> bool {
+        if (!ring_peek(seq, e)) return false;
+        // Issued only once the slot's value is in hand (the branch depends on
         // it), so the scheduler cannot overwrite the slot before this read.
-        if (e.code != kNoItem)
-            mbar_arrive_cluster_relaxed(mapa_shared(smem_u32(&item_empty[slot]), 1));
+        if (e.code != kNoItem && e.local >= 0) ring_free(seq);
         return true;
     };
     auto ring_job = [&](int seq) -> Job {
@@ -620,19 +630,26 @@ ns_gemm_kernel(const __grid_constant__ NsParams P) {
         if (lane == 0) {
             int si = 0;
             for (int seq = 0;; ++seq) {
-                const Job job = next_job(seq);
-                if (job.state == kJobTimeout) {
+                NsEntry e;
+                if (!ring_peek(seq, e)) {
                     raise_timeout(P, abort_flag, kSiteItem + 48, -2, seq);
                     break;
                 }
-                if (job.state == kJobEnd) break;
-                if (job.stage + 1 >= ns_num_stages(P, P.cls[job.w.cls])) continue;
-                if (!mbar_wait_bounded(&sig_bar[si % kSigSlots], (si / kSigSlots) & 1, budget, abort_flag)) {
-                    raise_timeout(P, abort_flag, kSiteSignal, job.local, seq);
-                    break;
+                if (e.g < 0) break;
+                const int stage = entry_stage(e);
+                const bool report = stage + 1 < ns_num_stages(P, P.cls[entry_cls(e)]);
+                if (report) {
+                    if (!mbar_wait_bounded(&sig_bar[si % kSigSlots], (si / kSigSlots) & 1, budget, abort_flag)) {
+                        raise_timeout(P, abort_flag, kSiteSignal, e.local, seq);
+                        break;
+                    }
+                    ++si;
                 }
-                ++si;
-                red_release_gpu_add(P.done + job.stage * P.nmat + job.g, kEpiWarps);
+                // Only now may the slot be published again: item seq + kItemSlots,
+                // whose reports would complete this phase of sig_bar a second
+                // time, cannot reach the epilogue before.
+                ring_free(seq);
+                if (report) red_release_gpu_add(P.done + stage * P.nmat + e.g, kEpiWarps);
             }
         }
     } else {
