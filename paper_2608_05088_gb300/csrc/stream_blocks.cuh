@@ -150,6 +150,15 @@ __device__ __forceinline__ void load8(const void* base, bool bf16, size_t off, f
     }
 }
 
+// 4 consecutive gradient elements (bf16 or fp32) at element offset off.
+__device__ __forceinline__ float4 load4_g(const void* base, bool bf16, size_t off) {
+    if (!bf16) return __ldg(reinterpret_cast<const float4*>(static_cast<const float*>(base) + off));
+    const uint2 u = __ldg(reinterpret_cast<const uint2*>(static_cast<const __nv_bfloat16*>(base) + off));
+    const float2 a = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162*>(&u.x));
+    const float2 b = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162*>(&u.y));
+    return make_float4(a.x, a.y, b.x, b.y);
+}
+
 __device__ __forceinline__ uint4 pack8_bf16(const float (&v)[8]) {
     uint4 u;
     __nv_bfloat162* h = reinterpret_cast<__nv_bfloat162*>(&u);
@@ -297,13 +306,12 @@ constexpr int kPreTileFloats = 2 * 64 * 64;
 // thread (four rows and two sub-tiles spilled at 4 blocks per SM and streamed
 // 7 % slower on GPT-2 Large, 14 % on a 16384 x 4096 matrix; one row at 6
 // blocks per SM was 2 % slower on GPT-2 Large and 5-10 % on wide stress
-// matrices).
+// matrices).  kMalter also sums (L G R)^2, G's loads issued with M's.
 constexpr int kPreBatch = 2;
 constexpr int kPreAhead = 1;
-template <bool kTall>
+template <bool kTall, bool kMalter>
 __device__ __forceinline__ void prescale_block(const MatDesc& d, const UserPtrs& up, int local,
-                                               int malter, int tid, float* tile,
-                                               float2* red) {
+                                               int tid, float* tile, float2* red) {
     constexpr int P = kLdPlain;
     const int m = d.m, n = d.n;
     // A tall matrix's blocks walk down a column band first, so the blocks
@@ -331,7 +339,7 @@ __device__ __forceinline__ void prescale_block(const MatDesc& d, const UserPtrs&
         const int row0 = r0 + warp * 8;
 #pragma unroll
         for (int rb = 0; rb < 8; rb += kPreBatch) {
-            float mv[kPreBatch][8], li[kPreBatch];
+            float mv[kPreBatch][8], gv[kPreBatch][8], li[kPreBatch];
             bool ok[kPreBatch];
 #pragma unroll
             for (int u = 0; u < kPreBatch; ++u) {
@@ -345,6 +353,7 @@ __device__ __forceinline__ void prescale_block(const MatDesc& d, const UserPtrs&
                     mv[u][0] = a.x; mv[u][1] = a.y; mv[u][2] = a.z; mv[u][3] = a.w;
                     mv[u][4] = b.x; mv[u][5] = b.y; mv[u][6] = b.z; mv[u][7] = b.w;
                     li[u] = ld_f<P>(Lv + row);
+                    if constexpr (kMalter) load8<kLdRO>(up.g, gbf, off, gv[u]);
                 }
             }
 #pragma unroll
@@ -359,12 +368,10 @@ __device__ __forceinline__ void prescale_block(const MatDesc& d, const UserPtrs&
                     s_mt = fmaf(v[j], v[j], s_mt);
                 }
                 *reinterpret_cast<uint4*>(d.X0 + off) = pack8_bf16(v);
-                if (malter) {
-                    float gv[8];
-                    load8<kLdRO>(up.g, gbf, off, gv);
+                if constexpr (kMalter) {
 #pragma unroll
                     for (int j = 0; j < 8; ++j) {
-                        const float a = li[u] * gv[j] * rj[j];
+                        const float a = li[u] * gv[u][j] * rj[j];
                         s_lgr = fmaf(a, a, s_lgr);
                     }
                 }
@@ -403,13 +410,21 @@ __device__ __forceinline__ void prescale_block(const MatDesc& d, const UserPtrs&
             float* __restrict__ tb = tile + (sub & 1) * (64 * 64);
             float4 R4 = make_float4(0.f, 0.f, 0.f, 0.f);
             if (col < n) R4 = ld_f4<P>(Rv + col);
+            float4 gq[4];
+            if constexpr (kMalter) {
+#pragma unroll
+                for (int pass = 0; pass < 4; ++pass) {
+                    const int row = r0 + pass * 16 + (t >> 4);
+                    gq[pass] = make_float4(0.f, 0.f, 0.f, 0.f);
+                    if (row < m && col < n) gq[pass] = load4_g(up.g, gbf, static_cast<size_t>(row) * n + col);
+                }
+            }
 #pragma unroll
             for (int pass = 0; pass < 4; ++pass) {
                 const int rr = pass * 16 + (t >> 4);
                 const int row = r0 + rr;
                 float v0 = 0.f, v1 = 0.f, v2 = 0.f, v3 = 0.f;
                 if (row < m && col < n) {
-                    const size_t off = static_cast<size_t>(row) * n + col;
                     const float Li = li[pass];
                     const float4 q = mq[sub % kPreAhead][pass];
                     v0 = Li * q.x * R4.x; v1 = Li * q.y * R4.y;
@@ -417,21 +432,9 @@ __device__ __forceinline__ void prescale_block(const MatDesc& d, const UserPtrs&
                     // explicit fused multiply-adds: the same rounding wherever
                     // this block is compiled
                     s_mt = fmaf(v3, v3, fmaf(v2, v2, fmaf(v1, v1, fmaf(v0, v0, s_mt))));
-                    if (malter) {
-                        float gq[4];
-                        if (gbf) {
-                            const uint2 u = *reinterpret_cast<const uint2*>(
-                                static_cast<const __nv_bfloat16*>(up.g) + off);
-                            const float2 a = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162*>(&u.x));
-                            const float2 b = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162*>(&u.y));
-                            gq[0] = a.x; gq[1] = a.y; gq[2] = b.x; gq[3] = b.y;
-                        } else {
-                            const float4 gf = *reinterpret_cast<const float4*>(
-                                static_cast<const float*>(up.g) + off);
-                            gq[0] = gf.x; gq[1] = gf.y; gq[2] = gf.z; gq[3] = gf.w;
-                        }
-                        const float a0 = Li * gq[0] * R4.x, a1 = Li * gq[1] * R4.y;
-                        const float a2 = Li * gq[2] * R4.z, a3 = Li * gq[3] * R4.w;
+                    if constexpr (kMalter) {
+                        const float a0 = Li * gq[pass].x * R4.x, a1 = Li * gq[pass].y * R4.y;
+                        const float a2 = Li * gq[pass].z * R4.z, a3 = Li * gq[pass].w * R4.w;
                         s_lgr = fmaf(a3, a3, fmaf(a2, a2, fmaf(a1, a1, fmaf(a0, a0, s_lgr))));
                     }
                 }

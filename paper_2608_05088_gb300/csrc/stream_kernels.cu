@@ -111,7 +111,9 @@ __global__ void __launch_bounds__(32 * kPadRows) pad_kernel(const __grid_constan
 // The streaming kernels' minimum resident blocks per SM (statistics 3,
 // prescale 5 for wide matrices and 4 for tall ones, apply 8) trade registers
 // for resident warps: more warps per SM kept more of HBM busy than more loads
-// in flight per thread did.
+// in flight per thread did.  MALTER's prescale also reads G: with G's loads issued
+// beside M's at one block per SM less, GPT-2 Medium's takes 478 us (6.3 TB/s)
+// where loading G after M's arithmetic took 510, and at 5 blocks 518.
 template <bool kStats>
 __global__ void __launch_bounds__(256, 3)
 stats_kernel(const MatDesc* __restrict__ mats, const UserPtrs* __restrict__ ptrs,
@@ -142,31 +144,30 @@ finalize_kernel(const MatDesc* __restrict__ mats, const UserPtrs* __restrict__ p
 // One launch for the wide matrices, one for the tall ones (their NS frame is
 // Mt^T, written through shared-memory transposes): ids lists the launch's
 // matrices and pref its block prefix.
-__global__ void __launch_bounds__(256, 5)
+template <bool kMalter>
+__global__ void __launch_bounds__(256, kMalter ? 4 : 5)
 prescale_wide_kernel(const MatDesc* __restrict__ mats, const UserPtrs* __restrict__ ptrs,
-                     const int32_t* __restrict__ ids, const int32_t* __restrict__ pref, int count,
-                     int malter) {
+                     const int32_t* __restrict__ ids, const int32_t* __restrict__ pref, int count) {
     __shared__ float2 red[8];
     chain_wait();
     const int32_t x = blockIdx.x;
     const int k = find_mat(pref, count, x);
     const int g = after_wait(__ldg(ids + k));
-    blk::prescale_block<false>(mats[g], ptrs[g], x - __ldg(pref + k), malter, threadIdx.x, nullptr,
-                               red);
+    blk::prescale_block<false, kMalter>(mats[g], ptrs[g], x - __ldg(pref + k), threadIdx.x, nullptr, red);
 }
 
-__global__ void __launch_bounds__(256, 4)
+template <bool kMalter>
+__global__ void __launch_bounds__(256, kMalter ? 3 : 4)
 prescale_tall_kernel(const MatDesc* __restrict__ mats, const UserPtrs* __restrict__ ptrs,
                      const int32_t* __restrict__ ids, const int32_t* __restrict__ pref, int count,
-                     int32_t base, int malter) {
+                     int32_t base) {
     __shared__ __align__(16) float tile[blk::kPreTileFloats];
     __shared__ float2 red[8];
     chain_wait();
     const int32_t x = base + static_cast<int32_t>(blockIdx.x);   // pref continues the wide launch's
     const int k = find_mat(pref, count, x);
     const int g = after_wait(__ldg(ids + k));
-    blk::prescale_block<true>(mats[g], ptrs[g], x - __ldg(pref + k), malter, threadIdx.x, tile,
-                              red);
+    blk::prescale_block<true, kMalter>(mats[g], ptrs[g], x - __ldg(pref + k), threadIdx.x, tile, red);
 }
 
 // ------------------------------------------------------------------ norms
@@ -266,13 +267,13 @@ cudaError_t launch_prescale(const MatDesc* mats, const UserPtrs* ptrs, const int
                             const int32_t* pref, int wide, int32_t wide_blocks, int tall,
                             int32_t tall_blocks, int malter, cudaStream_t s) {
     if (wide > 0 && wide_blocks > 0) {
-        const cudaError_t e = launch_chained(prescale_wide_kernel, wide_blocks, 256, 0, s, mats, ptrs, ids,
-                                             pref, wide, malter);
+        const cudaError_t e = launch_chained(malter ? prescale_wide_kernel<true> : prescale_wide_kernel<false>,
+                                             wide_blocks, 256, 0, s, mats, ptrs, ids, pref, wide);
         if (e != cudaSuccess) return e;
     }
     if (tall > 0 && tall_blocks > 0)
-        return launch_chained(prescale_tall_kernel, tall_blocks, 256, 0, s, mats, ptrs, ids + wide,
-                              pref + wide, tall, wide_blocks, malter);
+        return launch_chained(malter ? prescale_tall_kernel<true> : prescale_tall_kernel<false>, tall_blocks, 256,
+                              0, s, mats, ptrs, ids + wide, pref + wide, tall, wide_blocks);
     return cudaSuccess;
 }
 
