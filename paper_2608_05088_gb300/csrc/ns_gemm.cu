@@ -60,7 +60,7 @@
 //    items j, j + npairs, ...  The stream orders the stages.
 //  * Persistent: one launch for the whole run.  A scheduler thread per pair (the
 //    odd CTA's otherwise idle MMA-warp thread) claims items with an atomic on a
-//    global counter and publishes them to a 4-slot ring in both CTAs' shared
+//    global counter and publishes them to a 3-slot ring in both CTAs' shared
 //    memory (st.async messages on mbarriers).  Before it reads a tile's
 //    operands, each producer waits (bounded, acquire) until the previous stage
 //    of the tile's matrix is complete -- every epilogue warp of every tile of
@@ -123,10 +123,14 @@ constexpr uint32_t kStageOutBytes = 2 * kStoreBoxBytes * kEpiWarps;  // double-b
 constexpr size_t kSmemBytes =
     static_cast<size_t>(kStages) * Tile<kWideN>::kStageBytes + kStageOutBytes + 1024;
 constexpr uint16_t kPairMask = 0x3;
-// Persistent schedule: slots of the item ring (how far the scheduler may run
-// ahead of the slowest reader, the epilogue), and the readers of each slot:
-// both producers, the even CTA's MMA thread, every epilogue warp of both CTAs.
-constexpr int kItemSlots = 4;
+// Persistent schedule: slots of the item ring, and the readers of each slot: both
+// producers, the even CTA's MMA thread, every epilogue warp and the signal warp of
+// both CTAs.  A slot is free again once its tile has been reported, so a pair holds
+// at most this many claimed tiles: one in the epilogue, one in the MMAs, one in the
+// loads.  More are claimed by pairs that cannot start them yet while others idle:
+// GPT-2 Small's step takes 1120 us with 3, 1132 with 4 and 1170 with 6, but 1151
+// with 2; GPT-2 Medium and larger sets differ by less than 0.3 % between 3 and 6.
+constexpr int kItemSlots = 3;
 constexpr int kNoItem = -0x7fffffff;   // never stored in the ring
 constexpr uint32_t kItemReaders = 5 + 2 * kEpiWarps;
 static_assert(2 * kEpiWarps == static_cast<int>(kNsSignalsPerTile),
@@ -381,18 +385,18 @@ ns_gemm_kernel(const __grid_constant__ NsParams P) {
         const int slot = seq % kItemSlots;
         const uint32_t par = static_cast<uint32_t>(seq / kItemSlots) & 1u;
         if (!mbar_wait_cluster_bounded(&item_full[slot], par, budget, abort_flag)) return false;
-        const volatile int32_t* v = reinterpret_cast<const volatile int32_t*>(&item_ring[slot]);
-        e.code = v[0];
-        e.g = v[1];
-        e.local = v[2];
-        e.target = static_cast<uint32_t>(v[3]);
+        const int4 v = ld_shared_v4(&item_ring[slot]);
+        e.code = v.x;
+        e.g = v.y;
+        e.local = v.z;
+        e.target = static_cast<uint32_t>(v.w);
         return true;
     };
     auto ring_entry = [&](int seq, NsEntry& e) -> bool {
         if (!ring_peek(seq, e)) return false;
-        // Issued only once the slot's value is in hand (the branch depends on
-        // it), so the scheduler cannot overwrite the slot before this read.
-        if (e.code != kNoItem && e.local >= 0) ring_free(seq);
+        // Issued only once the slot's value is in hand (one load, and the branch
+        // depends on it), so the scheduler cannot overwrite the slot before this read.
+        if (e.code != kNoItem) ring_free(seq);
         return true;
     };
     auto ring_job = [&](int seq) -> Job {

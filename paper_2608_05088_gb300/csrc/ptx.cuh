@@ -144,7 +144,13 @@ __device__ __forceinline__ void st_async_v4(uint32_t cluster_addr, int32_t a, in
                  ::"r"(cluster_addr), "r"(a), "r"(b), "r"(c), "r"(d), "r"(cluster_bar) : "memory");
 }
 
-
+// One 16-byte load from shared memory (16-byte aligned), not moved or repeated.
+__device__ __forceinline__ int4 ld_shared_v4(const void* p) {
+    int4 v;
+    asm volatile("ld.volatile.shared.v4.b32 {%0, %1, %2, %3}, [%4];"
+                 : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "r"(smem_u32(p)) : "memory");
+    return v;
+}
 
 // --------------------------------------------- cross-CTA signals in global memory
 // Orders this thread's generic-proxy accesses of global memory with its
