@@ -266,6 +266,33 @@ def ncu_tensor_pipe():
         return None
 
 
+def ns_flops_run(wl, hp):
+    """(flops, issued flops) of the Newton-Schulz products that one step runs,
+    from the library's plan for each shape of the set.  flops counts a symmetric
+    product's upper triangle, issued the whole 256 x 256 tiles on and above its
+    diagonal.  The plan depends on the set's size through its number of 256 x 256
+    tiles, so each shape is asked for as many matrices as hold that many."""
+    from paper_2608_05088_gb300 import malt
+
+    def sym_tiles(p):
+        t = -(-p // 256)
+        return t * (t + 1) // 2
+
+    frames = [(min(s), max(s)) for s in wl.shapes]
+    total = sum(sym_tiles(p) for p, _ in frames)
+    run = issued = 0.0
+    for p, q in set(frames):
+        plan = malt.malt_ns_plan(p, q, -(-total // sym_tiles(p)), hp)
+        tp, tq = -(-p // 256), -(-q // 256)
+        one = one_issued = 0.0
+        for op in plan:
+            one += (1.0 * p * p * q, 1.0 * p ** 3, 2.0 * p * p * q)[op.kind]
+            one_issued += 2.0 * 256 ** 3 * (sym_tiles(p) * tq, sym_tiles(p) * tp, tp * tq * tp)[op.kind]
+        run += one * frames.count((p, q))
+        issued += one_issued * frames.count((p, q))
+    return run, issued
+
+
 def ncu_traffic_per_launch(persistent: bool):
     """DRAM bytes per NS GEMM launch (of the schedule the timed steps used)
     from the committed ncu summary, or None when a kernel source changed
@@ -459,7 +486,7 @@ def run_stress_sweep(args):
                     raise SystemExit(f"stress step failed: {wl.name}")
                 t_ms = e0.elapsed_time(e1) / args.steps
                 ns_ms = sum(prof[x][0] for x in malt.NS_KINDS) / args.steps
-                ns_tf = wl.ns_flops_min() / (ns_ms / 1e3) / 1e12
+                ns_tf = ns_flops_run(wl, hp)[0] / (ns_ms / 1e3) / 1e12
                 elems = wl.elements
                 mem = {}
                 for kind, bpe in (("stats", 12.0), ("prescale", 6.0), ("apply", 6.0)):
@@ -798,11 +825,11 @@ def run_malt(args):
     pk, pk_src = peaks()
     ns_ms = sum(prof[k][0] for k in malt.NS_KINDS)
     ns_launches = sum(prof[k][1] for k in malt.NS_KINDS)
-    # Algorithmic work: the Newton-Schulz flops with the symmetry of the Gram
-    # matrix and of the polynomial used (3 p^2 q + p^3 per matrix and iteration),
-    # which is what the kernels compute (upper-triangle tiles only).
-    flops = wl.ns_flops_min() * args.steps
-    achieved = flops / (ns_ms / 1e3) / 1e12
+    # Work counted: the products that the step runs (the library's own plan: wide
+    # frames merge iterations in p x p matrices, which takes fewer operations),
+    # each symmetric product as its upper triangle.
+    run_flops, run_issued = ns_flops_run(wl, hp)
+    achieved = run_flops * args.steps / (ns_ms / 1e3) / 1e12
     dense_equiv = wl.ns_flops_dense() * args.steps / (ns_ms / 1e3) / 1e12
     peak = float(pk["bf16_tflops_sustained"])
     persistent_timed = prof["ns_persistent"][1] > 0 and prof["ns_bx"][1] == 0
@@ -811,18 +838,21 @@ def run_malt(args):
         wl.name == "gpt2_large" and not args.layers) else None
     roofline = {"bound": "tensor", "achieved": achieved, "peak": peak, "unit": "TFLOP/s",
                 "frac": achieved / peak, "traffic": traffic,
-                "kernel": ("ns_gemm_kernel, persistent schedule (every Gram, Poly and BX "
-                           "product of the k iterations in one launch)"
+                "kernel": ("ns_gemm_kernel, persistent schedule (every product of the k "
+                           "iterations in one launch)"
                            if prof["ns_persistent"][1] > 0 else
-                           "ns_gemm_kernel, phased schedule (one launch per Gram, Poly and BX "
-                           "product)"),
+                           "ns_gemm_kernel, phased schedule (one launch per product)"),
                 "peak_source": f"{pk_src}: bf16_tflops_sustained",
-                "flops_per_step": wl.ns_flops_min(),
-                "flops_counted": "3p^2q + p^3 per matrix and NS iteration (symmetric Gram and polynomial)",
+                "flops_per_step": run_flops,
+                "flops_counted": "the products the step runs: p^2q per Gram, p^3 per p x p product "
+                                 "(both symmetric), 2p^2q per product with X",
+                # 3 p^2 q + p^3 per matrix and iteration: what the same step would
+                # take without merged iterations
+                "iterated_form_flops_per_step": wl.ns_flops_min(),
                 "dense_equivalent_tflops": dense_equiv,
                 # what the tensor cores execute: symmetric products as whole
                 # 256 x 256 tiles on and above the diagonal
-                "issued_tflops": wl.ns_flops_issued() * args.steps / (ns_ms / 1e3) / 1e12,
+                "issued_tflops": run_issued * args.steps / (ns_ms / 1e3) / 1e12,
                 "tensor_pipe_pct_ncu": ncu_tensor_pipe() if wl.name.startswith("gpt2_large") else None,
                 "launch_avg_ms": ns_ms / max(ns_launches, 1)}
     elems = wl.elements

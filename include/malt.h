@@ -250,11 +250,13 @@ int malt_profile_enable(malt_state_t* st, int32_t enable);
 int malt_profile_read(malt_state_t* st, double* ms_out, int64_t* launches_out, int32_t nkinds);
 
 /* Schedule of a state's steps (the Orth step of Algorithm 1 is k iterations
- * of A = X X^T, B' = aI + bA + cA^2, X <- B' X per matrix).
+ * of A = X X^T, B' = aI + bA + cA^2, X <- B' X per matrix; wide frames merge
+ * iterations, malt_ns_plan lists the products that run).
  *   MALT_NS_PHASED: one launch per HBM-bound stage (statistics, finalize,
  *     prescale, norms, scalars, apply) and one per Newton-Schulz product (3 k
- *     launches per group of up to 8 shape classes), each product over all
- *     matrices finished before the next starts.
+ *     launches per group of up to 8 shape classes, some more where iterations
+ *     are merged), each product over all matrices finished before the next
+ *     starts.
  *   MALT_NS_PERSISTENT: the same HBM-bound launches; one persistent launch
  *     per class group runs every product of every iteration.  Tiles are
  *     claimed dynamically in product order; a tile of matrix j waits on the
@@ -276,7 +278,8 @@ int malt_set_ns_schedule(malt_state_t* st, int32_t schedule);
 /* Host only (no GPU, no CUDA call): the work table of the persistent schedule
  * for these parameter shapes (only rows and cols are read) and ns_steps
  * iterations with every matrix in the iterated form (malt_ns_plan says which
- * form a matrix takes), in claim order, 8 int32 per item: launch group, stage (3 i +
+ * form a matrix takes) and tiles of 256 x 256 (sets of few tiles run narrower
+ * ones), in claim order, 8 int32 per item: launch group, stage (3 i +
  * kind for iteration i), kind (0 Gram, 1 Poly, 2 B*X), matrix index, local
  * index (the 256 x 256 tile of the NS frame; Gram and Poly list the upper
  * triangle only), the index of the counter the item waits for
