@@ -299,7 +299,7 @@ int malt_ns_schedule(const malt_param_t* params, int32_t n, int32_t ns_steps, in
  * iterates X; 4 holds Mt on the wide orientation, in bf16, at the start) and 6
  * (O), -1 for none; its operands are fp16 or bf16, its output is rounded to
  * fp16 or bf16.  kind 0 is a X X^T, 1 a product of two symmetric p x p
- * matrices (both kinds computed as an upper triangle and mirrored), 2 a product
+ * matrices (both kinds computed and stored as an upper triangle), 2 a product
  * of a p x p matrix with X.  Writes min(capacity, total) operations and the
  * total to *count.  MALT_ERR_INVALID_ARG for bad arguments,
  * MALT_ERR_UNSUPPORTED for a shape malt_init_state would reject. */

@@ -164,7 +164,7 @@ __host__ __device__ __forceinline__ int32_t entry_b(const NsEntry& e) {
 // the tensor maps of all its buffers.
 struct NsClass {  // 64-byte aligned through its CUtensorMap members
     CUtensorMap tmK[6];           // p x p buffers 0 .. 3 and the iterates X as K-major rows (box kBK x tile_n / 2)
-    CUtensorMap tmXmn[2];         // the iterates as an MN-major [K][N] operand (box kBMN x kBK)
+    CUtensorMap tmMn[6];          // the same buffers as an MN-major operand (box kBMN x kBK)
     CUtensorMap stK[6], stO;      // epilogue stores of the same buffers and of O: box 32 x 32, 64-byte swizzle
     CUtensorMap stOt;             // the O buffer as [q][p]: a tall W's O, stored in W's layout
     int32_t p, q, batch;

@@ -89,7 +89,7 @@ struct ShapeClass {
     __nv_bfloat16* O = nullptr;                  // last iterate, per matrix in W's layout:
                                                  // [p][q] (wide) or [q][p] (tall)
     int tile_n = kWideN;                         // width of the set's output tiles
-    CUtensorMap tmK[6] = {}, tmXmn[2];           // K-major boxes of tile_n / 2 rows; 64 x 64 MN boxes
+    CUtensorMap tmK[6] = {}, tmMn[6] = {};       // K-major boxes of tile_n / 2 rows; 64 x 64 MN boxes
     CUtensorMap stK[6] = {}, stO, stOt;         // epilogue store maps (stOt: O as [q][p])
 };
 
@@ -317,10 +317,10 @@ constexpr int kStatusWords = 8;
 // Tile width: 256 columns, or 128 for a set of few tiles (counted 256 wide, per
 // product).  There CTA pairs idle and a product takes its latency; half as wide, a
 // tile's MMAs and its epilogue (2.3 us of a product's 7.8) take half the time.
-// Newton-Schulz at k = 5, us per step, wide / narrow: one 256 x 512 matrix 118 / 85,
-// one 1280 x 1280 196 / 158, 16 of 256 x 2048 (16 symmetric and 128 B*X tiles)
-// 161 / 132, 8 of 768 x 768 (48 and 72) 172 / 144, one 2048 x 2048 (36 and 64)
-// 259 / 263, 8 of 1024 x 1024 (80 and 128) 205 / 244.  The wide tile loads a quarter
+// Newton-Schulz at k = 5, us per step, wide / narrow: one 256 x 512 matrix 118 / 84,
+// one 1280 x 1280 181 / 151, 16 of 256 x 2048 (16 symmetric and 128 B*X tiles)
+// 162 / 134, 8 of 768 x 768 (48 and 72) 162 / 141, one 2048 x 2048 (36 and 64)
+// 246 / 251, 8 of 1024 x 1024 (80 and 128) 193 / 225.  The wide tile loads a quarter
 // less per flop.  narrow_tiles false: 256 always (malt_ns_schedule's tables).
 constexpr int kNarrowMaxSym = 48, kNarrowMaxBx = 128;
 void build_classes(const malt_param_t* params, int n, bool narrow_tiles, std::vector<MatDesc>& hmats,
@@ -406,9 +406,9 @@ void plan_ns_groups(const std::vector<ShapeClass>& classes, int nmat, std::vecto
             NsClass& C = P.cls[j];
             for (int b = 0; b < 6; ++b) {
                 C.tmK[b] = S.tmK[b];
+                C.tmMn[b] = S.tmMn[b];
                 C.stK[b] = S.stK[b];
             }
-            for (int b = 0; b < 2; ++b) C.tmXmn[b] = S.tmXmn[b];
             C.can_group = S.can_group ? 1 : 0;
             C.stO = S.stO;
             C.stOt = S.stOt;
@@ -672,11 +672,12 @@ int plan_and_allocate(malt_state* st, const malt_param_t* params, int n) {
         // operation's business)
         for (int b = 0; b < 2; ++b) {
             ok &= encode_3d(&C.tmK[kBufX + b], C.X[b], C.q, C.p, C.batch, C.tile_n / 2);
-            ok &= encode_3d(&C.tmXmn[b], C.X[b], C.q, C.p, C.batch, kBK);
+            ok &= encode_3d(&C.tmMn[kBufX + b], C.X[b], C.q, C.p, C.batch, kBK);
             ok &= encode_store(&C.stK[kBufX + b], C.X[b], C.q, C.p, C.batch);
         }
         for (int b = 0; b < (C.can_group ? 4 : 2); ++b) {
             ok &= encode_3d(&C.tmK[b], C.P[b], C.p, C.p, C.batch, C.tile_n / 2);
+            ok &= encode_3d(&C.tmMn[b], C.P[b], C.p, C.p, C.batch, kBK);
             ok &= encode_store(&C.stK[b], C.P[b], C.p, C.p, C.batch);
         }
         ok &= encode_store(&C.stO, C.O, C.q, C.p, C.batch);

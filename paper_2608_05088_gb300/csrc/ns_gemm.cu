@@ -9,9 +9,9 @@
 // iteration of the iterated form is three of them:
 //   kGram  A  = X X^T               (M = N = p, K = q)    operands: rows of X, rows of X
 //   kPoly  B' = a I + b A + c A A   (M = N = p, K = p)    operands: rows of A, rows of A (A = A^T)
-// A and B' are symmetric, so those two phases compute only the tiles on and
-// above the diagonal and store each off-diagonal tile twice (as is and
-// transposed); the products are then exactly symmetric.
+// A and B' are symmetric, so those two phases compute and store only the tiles
+// on and above the diagonal.  Readers take what lies below it from the tile
+// above, transposed: the slice is loaded as an MN-major operand (slices_below).
 //   kBX    X' = B' X                (M = p, N = q, K = p) operands: rows of B', X read MN-major
 // so a X + (b A + c A A) X = B' X with the a X term folded into B' (its error
 // is that of the bf16 B it rides on).  The kBX B operand is X itself, read as
@@ -20,13 +20,13 @@
 // H) are kPoly operations on other buffers, in fp16; they commute with A, so
 // they are symmetric too and take the same path.  GPT-2 Large (36 layers, k = 5):
 // 17 products in 8.76 ms in place of 15 in 10.4 ms; one 16384 x 4096 matrix at
-// k = 8 2.89 in place of 4.27 ms.  The
+// k = 8 2.89 in place of 4.27 ms (both before symmetric tiles were stored once).  The
 // 1/(||Mt||_F + ns_eps) normalisation is folded into the first iteration's
 // epilogues (A scaled by k^2, X' by k).  The last product's epilogue writes O
 // in W's orientation and per-warp partial sums of O^2 and of D^2 with
 // D = L O R (Algorithm 1, D_t line) for the graft.  O is stored in W's layout:
-// a tall matrix's tiles go out transposed (the staging used for the mirror
-// of a symmetric tile), so the apply pass streams every matrix the same way.
+// a tall matrix's tiles go out transposed, so the apply pass streams every
+// matrix the same way.
 //
 // Work split.  A cluster of two CTAs (a CTA pair on two SMs) computes one
 // 256 x 256 output tile per turn (256 x 128 in sets of few tiles, build_classes): CTA r owns rows [128 r, 128 r + 128) of the
@@ -82,6 +82,7 @@
 #include <cstdint>
 #include <cstdio>
 #include <mutex>
+#include <type_traits>
 
 #include "chain.cuh"
 #include "common.cuh"
@@ -150,6 +151,8 @@ static_assert(kEpiWarps == 8, "epilogue layout assumes two warps per lane quarte
 struct Ops {
     const CUtensorMap* a;
     const CUtensorMap* b;
+    const CUtensorMap* a_mn;    // the same buffers as MN-major operands
+    const CUtensorMap* b_mn;
     const CUtensorMap* out;
     int M, N, K;
 };
@@ -158,10 +161,20 @@ __device__ __forceinline__ Ops item_operands(const NsParams& P, const NsWork& w)
     const NsClass& C = P.cls[w.cls];
     const NsOp& o = w.op;
     const bool bx = o.kind == kBX;
-    return Ops{&C.tmK[o.a], bx ? &C.tmXmn[o.b - kBufX] : &C.tmK[o.b],
+    return Ops{&C.tmK[o.a], &C.tmK[o.b], &C.tmMn[o.a], &C.tmMn[o.b],
                o.out == kBufO ? &C.stO : &C.stK[o.out],
                C.p, bx ? C.q : C.p, o.kind == kGram ? C.q : C.p};
 }
+
+// A symmetric p x p buffer holds its 256 x 256 tiles on and above the diagonal.
+// The reduction slices of operand rows in tile row `row` that lie below it are the
+// first ones; their elements [r][k] are read as [k][r], MN-major instead of
+// K-major.  Storing every such tile a second time, transposed, cost the epilogue
+// (shuffles, a second staged box and store per chunk) more than these reads cost the
+// loads and the MMAs, at every size: Newton-Schulz of GPT-2 Small 742 -> 711 us, of
+// GPT-2 Medium 3050 -> 2932, one 4096 x 4096 matrix 894 -> 863, one 512 x 512 102 -> 96.
+__device__ __forceinline__ int slices_below(int row) { return row * (kTileM / kBK); }
+static_assert(kTileM / kBK % kGroup == 0, "the slices of a ring stage are read alike");
 
 // Bytes CTA `rank` loads for one reduction slice of a tile.  Boxes that lie
 // wholly past M or N are skipped: they only feed accumulator rows / columns
@@ -184,6 +197,26 @@ __device__ __forceinline__ uint32_t slice_bytes(const Ops& op, const NsWork& w, 
     }
     *nbox_b = nb;
     return bytes;
+}
+
+// Layout of an operand in its slot.
+using Mn = std::integral_constant<bool, true>;
+using Kn = std::integral_constant<bool, false>;
+
+// The MMAs of one reduction slice (kb-th of its tile), each operand K-major or
+// MN-major; idesc is that of two K-major operands.
+template <bool kAMn, bool kBMn>
+__device__ __forceinline__ void issue_slice(uint32_t d_tmem, uint32_t sa, bool same_ab, uint32_t idesc, int kb) {
+    const uint32_t sb = same_ab ? sa : sa + kABytes;
+    const uint64_t da = kAMn ? smem_desc_mn_sw128(sa, kMnLbo) : smem_desc_k_sw128(sa);
+    const uint64_t db = kBMn ? smem_desc_mn_sw128(sb, kMnLbo) : smem_desc_k_sw128(sb);
+    // Per 16-element MMA slice (addresses encoded >> 4): +32 bytes along K, or
+    // +16 K-rows = two 1024-byte atoms.
+    constexpr uint32_t kStepA = kAMn ? 2048u >> 4 : 2u, kStepB = kBMn ? 2048u >> 4 : 2u;
+#pragma unroll
+    for (int kk = 0; kk < kBK / 16; ++kk)
+        tc_mma_16bit_pair(d_tmem, da + kStepA * kk, db + kStepB * kk, idesc | idesc_majors(kAMn, kBMn),
+                          (kb | kk) != 0 ? 1u : 0u);
 }
 
 // Two floats <-> two 16-bit values (fp16 or bf16, round to nearest even).
@@ -340,7 +373,7 @@ ns_gemm_kernel(const __grid_constant__ NsParams P) {
             const NsClass& C = P.cls[c];
             for (int j = 0; j < 2; ++j) {
                 tma_prefetch_desc(&C.tmK[kBufX + j]);
-                tma_prefetch_desc(&C.tmXmn[j]);
+                tma_prefetch_desc(&C.tmMn[kBufX + j]);
             }
             for (int j = 0; j < (C.grouped ? 4 : 2); ++j) tma_prefetch_desc(&C.tmK[j]);
         }
@@ -497,35 +530,50 @@ ns_gemm_kernel(const __grid_constant__ NsParams P) {
                 const bool load_a = w.mt * kTileM + rank * kBM < op.M;
                 const int a_row = w.mt * kTileM + rank * kBM;
                 const int n0 = w.nt * kN + rank * kHalfN;
-                bool ok = true;
-                for (int k0 = 0; k0 < nkb; k0 += kGroup) {
-                    if (!mbar_wait_cluster_bounded(&empty_bar[stage], phase ^ 1u, budget, abort_flag)) {
-                        raise_timeout(P, abort_flag, kSiteStage, item, k0);
-                        ok = false;
-                        break;
-                    }
-                    const int nsub = min(kGroup, nkb - k0);
-                    const uint32_t fb = mapa_shared(smem_u32(&full_bar[stage]), 0);
-                    if (leader) mbar_arrive_expect_tx(&full_bar[stage], nsub * bytes_pair);
-                    for (int j = 0; j < nsub; ++j) {
-                        const int kb = k0 + j;
-                        uint8_t* sa = smem + (stage * kGroup + j) * kStageBytes;
-                        if (load_a) {
+                const int a_below = w.op.kind != kGram ? slices_below(w.mt) : 0;
+                const int b_below = b_mn ? nkb : w.op.kind == kPoly ? slices_below(w.nt * kN / kTileM) : 0;
+                // MN-major boxes of a slice of B (a half is counted whole where it is
+                // read from above the diagonal: boxes past N arrive as zeros)
+                const int nb_mn = b_mn ? nb_self : nb_self > 0 ? kHalfN / kBMN : 0;
+                // Slices [from, to), each operand K-major or MN-major.
+                auto load_slices = [&](auto a_mn, auto b_mn_, int from, int to) -> bool {
+                    for (int k0 = from; k0 < to; k0 += kGroup) {
+                        if (!mbar_wait_cluster_bounded(&empty_bar[stage], phase ^ 1u, budget, abort_flag)) {
+                            raise_timeout(P, abort_flag, kSiteStage, item, k0);
+                            return false;
+                        }
+                        const int nsub = min(kGroup, to - k0);
+                        const uint32_t fb = mapa_shared(smem_u32(&full_bar[stage]), 0);
+                        if (leader) mbar_arrive_expect_tx(&full_bar[stage], nsub * bytes_pair);
+                        for (int j = 0; j < nsub; ++j) {
+                            const int kx = (k0 + j) * kBK;
+                            uint8_t* sa = smem + (stage * kGroup + j) * kStageBytes;
+                            if (load_a) {
+                                if constexpr (decltype(a_mn)::value) {
 #pragma unroll
-                            for (int h = 0; h < kBM; h += kHalfN)
-                                tma_load_3d_pair(sa + h * (kBK * 2), op.a, kb * kBK, a_row + h, w.b, fb);
+                                    for (int h = 0; h < kBM; h += kBMN)
+                                        tma_load_3d_pair(sa + h * (kBK * 2), op.a_mn, a_row + h, kx, w.b, fb);
+                                } else {
+#pragma unroll
+                                    for (int h = 0; h < kBM; h += kHalfN)
+                                        tma_load_3d_pair(sa + h * (kBK * 2), op.a, kx, a_row + h, w.b, fb);
+                                }
+                            }
+                            if constexpr (decltype(b_mn_)::value) {
+                                for (int jb = 0; jb < nb_mn; ++jb)
+                                    tma_load_3d_pair(sa + kABytes + jb * kMnBoxBytes, op.b_mn, n0 + jb * kBMN, kx,
+                                                     w.b, fb);
+                            } else if (nb_self > 0) {
+                                tma_load_3d_pair(sa + kABytes, op.b, kx, n0, w.b, fb);
+                            }
                         }
-                        if (b_mn) {
-                            for (int jb = 0; jb < nb_self; ++jb)
-                                tma_load_3d_pair(sa + kABytes + jb * kMnBoxBytes, op.b,
-                                                 n0 + jb * kBMN, kb * kBK, w.b, fb);
-                        } else if (nb_self > 0) {
-                            tma_load_3d_pair(sa + kABytes, op.b, kb * kBK, n0, w.b, fb);
-                        }
+                        if (!leader) mbar_arrive_cluster_relaxed(fb);
+                        if (++stage == kRing) { stage = 0; phase ^= 1u; }
                     }
-                    if (!leader) mbar_arrive_cluster_relaxed(fb);
-                    if (++stage == kRing) { stage = 0; phase ^= 1u; }
-                }
+                    return true;
+                };
+                const bool ok = load_slices(Mn{}, Mn{}, 0, a_below) && load_slices(Kn{}, Mn{}, a_below, b_below) &&
+                                load_slices(Kn{}, Kn{}, b_below, nkb);
                 if (!ok) break;
             }
         }
@@ -571,11 +619,11 @@ ns_gemm_kernel(const __grid_constant__ NsParams P) {
                 const bool b_mn = w.op.kind == kBX;
                 const bool same_ab = kN == kTileM && w.op.a == w.op.b && w.mt == w.nt;
                 const int K = w.op.kind == kGram ? P.cls[w.cls].q : P.cls[w.cls].p;
-                const uint32_t idesc = b_mn ? (w.op.f16 ? idesc_16bit_f32(kTileM, kN, true, true)
-                                                        : idesc_16bit_f32(kTileM, kN, false, true))
-                                            : (w.op.f16 ? idesc_16bit_f32(kTileM, kN, true, false)
-                                                        : idesc_16bit_f32(kTileM, kN, false, false));
                 const int nkb = (K + kBK - 1) / kBK;
+                const int a_below = w.op.kind != kGram ? slices_below(w.mt) : 0;
+                const int b_below = b_mn ? nkb : w.op.kind == kPoly ? slices_below(w.nt * kN / kTileM) : 0;
+                const uint32_t idesc = w.op.f16 ? idesc_16bit_f32(kTileM, kN, true)
+                                                : idesc_16bit_f32(kTileM, kN, false);
                 const uint32_t acc = gi & 1, acc_phase = (gi >> 1) & 1;
                 ++gi;
                 if (!mbar_wait_cluster_bounded(&tempty_bar[acc], acc_phase ^ 1u, budget, abort_flag)) {
@@ -584,40 +632,27 @@ ns_gemm_kernel(const __grid_constant__ NsParams P) {
                 }
                 tc_fence_after();
                 const uint32_t d_tmem = tmem_base + acc * kN;
-                bool ok = true;
-                for (int k0 = 0; k0 < nkb; k0 += kGroup) {
-                    if (!mbar_wait_cluster_bounded(&full_bar[stage], phase, budget, abort_flag)) {
-                        raise_timeout(P, abort_flag, kSiteStageFull, item, k0);
-                        ok = false;
-                        break;
-                    }
-                    tc_fence_after();
-                    const int nsub = min(kGroup, nkb - k0);
-                    for (int j = 0; j < nsub; ++j) {
-                        const int kb = k0 + j;
-                        const uint32_t sa = smem_u32(smem + (stage * kGroup + j) * kStageBytes);
-                        const uint64_t da = smem_desc_k_sw128(sa);
-                        if (b_mn) {
-                            const uint64_t db = smem_desc_mn_sw128(sa + kABytes, kMnLbo);
-#pragma unroll
-                            for (int kk = 0; kk < kBK / 16; ++kk) {
-                                // A: +32 bytes along K; B: +16 K-rows = two 1024-byte atoms.
-                                tc_mma_16bit_pair(d_tmem, da + 2 * kk, db + (2048u >> 4) * kk,
-                                                  idesc, (kb | kk) != 0 ? 1u : 0u);
-                            }
-                        } else {
-                            const uint64_t db = smem_desc_k_sw128(same_ab ? sa : sa + kABytes);
-#pragma unroll
-                            for (int kk = 0; kk < kBK / 16; ++kk) {
-                                // +32 bytes along K per 16-element MMA slice (encoded >> 4).
-                                tc_mma_16bit_pair(d_tmem, da + 2 * kk, db + 2 * kk, idesc,
-                                                  (kb | kk) != 0 ? 1u : 0u);
-                            }
+                // Slices [from, to): with each form a loop of its own, the descriptors'
+                // steps and the instruction descriptor are constants (one loop that
+                // picks the form per ring stage was 3 - 6 % slower on 4096 x 4096).
+                auto issue_slices = [&](auto a_mn, auto b_mn_, int from, int to) -> bool {
+                    for (int k0 = from; k0 < to; k0 += kGroup) {
+                        if (!mbar_wait_cluster_bounded(&full_bar[stage], phase, budget, abort_flag)) {
+                            raise_timeout(P, abort_flag, kSiteStageFull, item, k0);
+                            return false;
                         }
+                        tc_fence_after();
+                        const int nsub = min(kGroup, to - k0);
+                        for (int j = 0; j < nsub; ++j)
+                            issue_slice<decltype(a_mn)::value, decltype(b_mn_)::value>(
+                                d_tmem, smem_u32(smem + (stage * kGroup + j) * kStageBytes), same_ab, idesc, k0 + j);
+                        tc_commit_pair_multicast(&empty_bar[stage], kPairMask);
+                        if (++stage == kRing) { stage = 0; phase ^= 1u; }
                     }
-                    tc_commit_pair_multicast(&empty_bar[stage], kPairMask);
-                    if (++stage == kRing) { stage = 0; phase ^= 1u; }
-                }
+                    return true;
+                };
+                const bool ok = issue_slices(Mn{}, Mn{}, 0, a_below) && issue_slices(Kn{}, Mn{}, a_below, b_below) &&
+                                issue_slices(Kn{}, Kn{}, b_below, nkb);
                 if (!ok) break;
                 tc_commit_pair_multicast(&tfull_bar[acc], kPairMask);
             }
@@ -705,7 +740,6 @@ ns_gemm_kernel(const __grid_constant__ NsParams P) {
             const bool in16 = op.f16 != 0, out16 = op.out16 != 0;
             const int M = C.p, N = op.kind == kBX ? C.q : C.p;
             const CUtensorMap* out_map0 = item_operands(P, w).out;
-            const bool sym = op.kind != kBX;
             const int row = w.mt * kTileM + rank * kBM + quarter * 32 + lane;
             const bool rok = row < M;
             const int g = job.g >= 0 ? job.g : C.mat_of[w.b];
@@ -843,9 +877,8 @@ ns_gemm_kernel(const __grid_constant__ NsParams P) {
                     }
                     obuf ^= 1;
                 }
-                if (store_t || (sym && w.nt * kN >= (w.mt + 1) * kTileM)) {
-                    // Mirror an off-diagonal tile of the symmetric product, or
-                    // store a tall matrix's O in W's layout: the transposed chunk
+                if (store_t) {
+                    // A tall matrix's O goes out in W's layout: the transposed chunk
                     // (box row = column j, 32 rows of this warp) goes to rows
                     // [col0, col0+32) x columns [row0, row0+32) of the map.
                     // Lane pairs swap the packed word of each column pair, and

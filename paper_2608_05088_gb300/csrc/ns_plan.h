@@ -88,14 +88,15 @@ inline bool ns_grouped_run(int k, double a, double b, double c) {
 
 // Frames that take the grouped form when the run may.  A merged iteration
 // replaces 3 p^2 q + p^3 by 4 p^3, which are equal at q = p, in more and less
-// efficient products (a p x p tile stores twice what it computes): at q = 1.5 p
-// the two forms take the same time, so q >= 2 p.  Where a set is only a few
+// efficient products (short reductions): at q = 1.5 p it gains 2 - 3 % in large
+// sets and loses 2 - 4 % in small ones (1280 x 1920, iterated / grouped: 32 of them
+// 1259 / 1230 us, 8 of them 369 / 386), so q >= 2 p.  Where a set is only a few
 // tiles, a product takes its latency plus its reduction, and the grouped form has
 // two products more: it pays once the q - 2 p that a merged iteration saves are
 // long enough or the set is large.  Measured at k = 5, us of Newton-Schulz per
-// step, iterated / grouped: one 512 x 1024 113 / 122, 32 of them 208 / 218, one
-// 512 x 2048 135 / 135, one 256 x 4096 158 / 134, 16 of 1024 x 2048 456 / 432,
-// one 2048 x 4096 451 / 428, 8 of 1280 x 5120 733 / 588.
+// step, iterated / grouped: one 512 x 1024 108 / 114, 32 of them 204 / 206, one
+// 512 x 2048 127 / 128, one 256 x 4096 155 / 133, 16 of 1024 x 2048 439 / 400,
+// one 2048 x 4096 383 / 339, 8 of 1280 x 5120 727 / 570.
 // tiles: 256 x 256 tiles of one symmetric product over the set.
 inline bool ns_grouped_shape(int64_t p, int64_t q, int64_t tiles) {
     return q >= 2 * p && 50 * (q - 2 * p) + tiles * p >= 50000;

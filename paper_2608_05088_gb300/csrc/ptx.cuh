@@ -351,14 +351,18 @@ __device__ __forceinline__ uint64_t smem_desc_mn_sw128(uint32_t smem_addr, uint3
     return d;
 }
 
-// Instruction descriptor for kind::f16: fp32 accumulator, bf16 A and B, both
-// K-major, shape M x N.
+// Instruction descriptor for kind::f16: fp32 accumulator, A and B both bf16 or
+// both fp16, both K-major, shape M x N.
 //   bits 4-5 D format (1 = f32), 7-9 A format (1 = bf16, 0 = f16), 10-12 B format (the same),
 //   bit 15/16 A/B major (0 = K), bits 17-22 N >> 3, bits 24-28 M >> 4.
-__host__ __device__ constexpr uint32_t idesc_16bit_f32(uint32_t M, uint32_t N, bool f16, bool b_mn_major) {
+__host__ __device__ constexpr uint32_t idesc_16bit_f32(uint32_t M, uint32_t N, bool f16) {
     const uint32_t fmt = f16 ? 0u : 1u;
-    return (1u << 4) | (fmt << 7) | (fmt << 10) | ((b_mn_major ? 1u : 0u) << 16) |
-           ((N >> 3) << 17) | ((M >> 4) << 24);
+    return (1u << 4) | (fmt << 7) | (fmt << 10) | ((N >> 3) << 17) | ((M >> 4) << 24);
+}
+
+// The bits that make an operand MN-major.
+__host__ __device__ constexpr uint32_t idesc_majors(bool a_mn, bool b_mn) {
+    return (a_mn ? 1u << 15 : 0u) | (b_mn ? 1u << 16 : 0u);
 }
 
 }  // namespace malt
