@@ -160,6 +160,9 @@ __host__ __device__ __forceinline__ int32_t entry_b(const NsEntry& e) {
     return static_cast<int32_t>(static_cast<uint32_t>(e.code) >> 16);
 }
 
+// Row stride of a p x p buffer: whole 32-byte sectors, which the epilogue loads at once.
+__host__ __device__ __forceinline__ int32_t ns_ld(int32_t p) { return (p + 15) / 16 * 16; }
+
 // One shape class (every matrix whose NS frame is p x q, stored batched) with
 // the tensor maps of all its buffers.
 struct NsClass {  // 64-byte aligned through its CUtensorMap members
@@ -176,7 +179,7 @@ struct NsClass {  // 64-byte aligned through its CUtensorMap members
     int32_t grouped;              // this run's form
     int32_t bx_col_major;         // list B*X tiles column by column (X larger than kBxColBytes)
     const int32_t* mat_of;        // [batch] -> matrix index
-    const uint16_t* A;            // p x p buffer 0 [batch][p][p], 16-bit (read by the H epilogue)
+    const uint16_t* A;            // p x p buffer 0 [batch][p][ns_ld(p)], 16-bit (read by the H epilogue)
 };
 
 // Work list of one launch.  Each class runs its form's operations in order

@@ -56,13 +56,13 @@ bool get_encoder() {
     return true;
 }
 
-// 3-D bf16 tensor [batch][rows][cols], box box_cols x box_rows x 1, zero fill
+// 3-D bf16 tensor [batch][rows][cols] with rows of ld elements, box box_cols x box_rows x 1, zero fill
 // outside the tensor on loads (stores skip the outside).
 bool encode_3d(CUtensorMap* map, const void* base, uint64_t cols, uint64_t rows, uint64_t batch,
-               uint32_t box_rows, uint32_t box_cols = kBK,
+               uint64_t ld, uint32_t box_rows, uint32_t box_cols = kBK,
                CUtensorMapSwizzle swizzle = CU_TENSOR_MAP_SWIZZLE_128B) {
     const cuuint64_t dims[3] = {cols, rows, batch};
-    const cuuint64_t strides[2] = {cols * 2, rows * cols * 2};
+    const cuuint64_t strides[2] = {ld * 2, rows * ld * 2};
     const cuuint32_t box[3] = {box_cols, box_rows, 1};
     const cuuint32_t estr[3] = {1, 1, 1};
     const CUresult r = g_encode(map, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 3, const_cast<void*>(base),
@@ -73,8 +73,9 @@ bool encode_3d(CUtensorMap* map, const void* base, uint64_t cols, uint64_t rows,
 }
 
 // Store map of an epilogue output: 32 x 32 boxes with 64-byte swizzle.
-bool encode_store(CUtensorMap* map, const void* base, uint64_t cols, uint64_t rows, uint64_t batch) {
-    return encode_3d(map, base, cols, rows, batch, 32, 32, CU_TENSOR_MAP_SWIZZLE_64B);
+bool encode_store(CUtensorMap* map, const void* base, uint64_t cols, uint64_t rows, uint64_t batch,
+                  uint64_t ld) {
+    return encode_3d(map, base, cols, rows, batch, ld, 32, 32, CU_TENSOR_MAP_SWIZZLE_64B);
 }
 
 struct ShapeClass {
@@ -515,7 +516,7 @@ int plan_and_allocate(malt_state* st, const malt_param_t* params, int n) {
     for (int k = 0; k < nc; ++k) {
         const ShapeClass& C = st->classes[k];
         const size_t pq = static_cast<size_t>(C.batch) * C.p * C.q * 2;
-        const size_t pp = static_cast<size_t>(C.batch) * C.p * C.p * 2;
+        const size_t pp = static_cast<size_t>(C.batch) * C.p * ns_ld(C.p) * 2;
         o_X0[k] = cv.take(pq);
         o_X1[k] = cv.take(pq);
         for (int j = 0; j < (C.can_group ? 4 : 2); ++j) o_P[j][k] = cv.take(pp);
@@ -671,17 +672,18 @@ int plan_and_allocate(malt_state* st, const malt_param_t* params, int n) {
         // (a map moves 16-bit elements; whether they are bf16 or fp16 is the
         // operation's business)
         for (int b = 0; b < 2; ++b) {
-            ok &= encode_3d(&C.tmK[kBufX + b], C.X[b], C.q, C.p, C.batch, C.tile_n / 2);
-            ok &= encode_3d(&C.tmMn[kBufX + b], C.X[b], C.q, C.p, C.batch, kBK);
-            ok &= encode_store(&C.stK[kBufX + b], C.X[b], C.q, C.p, C.batch);
+            ok &= encode_3d(&C.tmK[kBufX + b], C.X[b], C.q, C.p, C.batch, C.q, C.tile_n / 2);
+            ok &= encode_3d(&C.tmMn[kBufX + b], C.X[b], C.q, C.p, C.batch, C.q, kBK);
+            ok &= encode_store(&C.stK[kBufX + b], C.X[b], C.q, C.p, C.batch, C.q);
         }
         for (int b = 0; b < (C.can_group ? 4 : 2); ++b) {
-            ok &= encode_3d(&C.tmK[b], C.P[b], C.p, C.p, C.batch, C.tile_n / 2);
-            ok &= encode_3d(&C.tmMn[b], C.P[b], C.p, C.p, C.batch, kBK);
-            ok &= encode_store(&C.stK[b], C.P[b], C.p, C.p, C.batch);
+            const uint64_t ld = ns_ld(C.p);
+            ok &= encode_3d(&C.tmK[b], C.P[b], C.p, C.p, C.batch, ld, C.tile_n / 2);
+            ok &= encode_3d(&C.tmMn[b], C.P[b], C.p, C.p, C.batch, ld, kBK);
+            ok &= encode_store(&C.stK[b], C.P[b], C.p, C.p, C.batch, ld);
         }
-        ok &= encode_store(&C.stO, C.O, C.q, C.p, C.batch);
-        ok &= encode_store(&C.stOt, C.O, C.p, C.q, C.batch);
+        ok &= encode_store(&C.stO, C.O, C.q, C.p, C.batch, C.q);
+        ok &= encode_store(&C.stOt, C.O, C.p, C.q, C.batch, C.p);
         if (!ok) {
             std::fprintf(stderr, "malt: cuTensorMapEncodeTiled failed for class %d x %d\n", C.p, C.q);
             return MALT_ERR_CUDA;
