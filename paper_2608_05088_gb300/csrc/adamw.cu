@@ -13,7 +13,7 @@
 // One grouped launch covers every tensor of a step: block b takes a
 // contiguous run of kAdamChunk elements of one tensor (a block-prefix table
 // maps blocks to tensors).  Each thread streams 4 elements per 128-bit load
-// of w, m, v and g (64-bit for a bf16 gradient), two such groups in flight.
+// of w, m, v and g (64-bit for a bf16 gradient), one such group in flight.
 // The update is 30 B/elem of HBM traffic with an fp32 gradient and a bf16
 // copy (g 4, w 4+4, m 4+4, v 4+4, copy 2).  A tiny bind launch before it
 // copies the caller's pointers to the device and advances t, so the step

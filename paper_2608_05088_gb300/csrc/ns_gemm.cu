@@ -582,9 +582,9 @@ ns_gemm_kernel(const __grid_constant__ NsParams P) {
             // ------------------------------------------ scheduler (odd CTA)
             // Claim items in table order and publish them up to kItemSlots ahead
             // of the slowest reader.  The next item is claimed only once the
-            // last one can run: claimed at once, five items a pair left a stage
-            // of 136 tiles to 28 of the 76 pairs (one 4096 x 4096 matrix 916 us
-            // -> 1245).
+            // last one can run: claimed at once, five items a pair (with a ring of
+            // four slots) left a stage of 136 tiles to 28 of the 76 pairs (one
+            // 4096 x 4096 matrix 916 us -> 1245).
             for (int seq = 0;; ++seq) {
                 NsEntry e = claim_next();
                 const uint32_t target = e.target;
