@@ -14,17 +14,28 @@
 //    symmetric themselves, and every one is computed as an upper triangle.
 //    With q = 4 p a merged iteration costs 4 p^3 in place of 13 p^3.
 //
-// Rounding.  In bf16 the grouped form loses accuracy (A carries the squared
-// singular values), so from the second iterate on it works in fp16: 11
-// significant bits in place of 8.  The iterates are bounded (|p(x)| stays near
-// 1), so the range is known: X is stored times kScaleX and A times kScaleA
-// (powers of two), which puts fp16's smallest step 2^-24 at 2^-32 and 2^-34 of
-// a unit singular value.  The first iteration keeps bf16, because Mt's scale is
-// not known before it.  Against fp64 the grouped form is closer than the
-// iterated one: 0.30-0.55e-2 in place of 0.7-1.7e-2 relative on frames with
-// log-normal scales (sigma 0 to 3, k = 5), and no worse on the geometric,
-// low-rank and graded spectra of tests/test_ns_plan.py, which reads the plan
-// from the library and runs its arithmetic on the CPU.
+// Rounding.  X stays in bf16 in both forms: its rows and columns may differ by many
+// decades (a frame that is not preconditioned, rows without gradients), and bf16 has
+// fp32's range.  With X in fp16, whatever its scale, a column 1e-10 of the others
+// left with an error of 1.  The p x p matrices of a group are fp16, 11 significant
+// bits in place of 8: in bf16 the grouped form loses accuracy, since A carries the
+// squared singular values (1.5 times the iterated form's error, 2 in the worst row).
+// Their entries are bounded (|p(x)| stays near 1), so each is stored times the
+// power of two that puts its bound at 2^15 (ns_grouped_run): an entry of A keeps
+// all its bits down to 2^-28 of a unit singular value squared, one of H down to
+// 2^-27.  What is left of the range: the entries that couple a small row of X with the
+// others are that small where the row is below 1e-8 of the frame.  With half the rows
+// scaled by 1e-8 nothing is lost (0.004 - 0.011 in those rows, iterated 0.009 - 0.018);
+// by 1e-9 it is 0.005 - 0.08, by 1e-10 0.007 - 0.7, by 1e-12 they keep only the leading
+// factor a^k.  The running product that is applied to X goes out in bf16, X's type.
+//
+// Against fp64, k = 4 to 8, relative to the iterated form's error on frames with
+// log-normal scales (sigma 0 to 3, as they are and preconditioned): the whole frame
+// 0.6 - 0.9, the median row and column 0.5 - 0.9, the worst row and column 0.4 - 0.95
+// (geometric means over shapes 64 x 128 to 512 x 2048).  At k = 3 the worst column is
+// 1.0 - 1.3, so 3 iterations stay iterated.  tests/test_ns_plan.py reads the plan from
+// the library and runs its arithmetic on the CPU, on these frames and on geometric,
+// low-rank, graded and blocked ones.
 //
 // Which form runs (ns_grouped_run, ns_grouped_shape) follows from k, from the
 // coefficients, from the shape and from the size of the set.
@@ -36,27 +47,36 @@
 
 namespace malt {
 
-// Groups of a k-iteration run after the first iteration (k = 3 .. 8), zero
+// Groups of a k-iteration run after the first iteration (k = 4 .. 8), zero
 // ended.  Pairs; three at a time loses accuracy on ill-conditioned frames, so
 // it is taken only where it ends the longest run.
-constexpr int kMinGroupedSteps = 3, kMaxGroupedSteps = 8;
+constexpr int kMinGroupedSteps = 4, kMaxGroupedSteps = 8;
 constexpr int kNsGroups[kMaxGroupedSteps + 1][4] = {
-    {0}, {0}, {0}, {2, 0}, {2, 1, 0}, {2, 2, 0}, {2, 2, 1, 0}, {2, 2, 2, 0}, {2, 2, 3, 0}};
+    {0}, {0}, {0}, {0}, {2, 1, 0}, {2, 2, 0}, {2, 2, 1, 0}, {2, 2, 2, 0}, {2, 2, 3, 0}};
 
-constexpr float kScaleX = 256.f;      // fp16 iterates hold kScaleX * X
-constexpr float kScaleA = 1024.f;     // fp16 Gram matrices hold kScaleA * A (and H A the same)
+// Factors (powers of two) by which a group's fp16 matrices are stored.
+struct NsScales {
+    float a = 1.f, h = 1.f, ha = 1.f, q = 1.f;   // A, H, H A, and a running product that grows further
+};
+
+// The power of two that brings a bound to at most 2^15, half of fp16's largest
+// value: rounding moves what the bounds say by a few percent at most.
+inline float ns_scale_to_fp16(double bound) {
+    return static_cast<float>(std::exp2(std::floor(15.0 - std::log2(std::fmax(bound, 1.0)))));
+}
 
 // Whether a run of k iterations with these coefficients may take the grouped
-// form: the fp16 values must stay in range and above its smallest step.  The
+// form, and its scales: the fp16 values must stay in range.  The
 // singular values of the first iterate are at most 1 (X is divided by its
 // Frobenius norm), so the range of every later one follows from the extrema of
-// x h(x^2), h(t) = a + b t + c t^2.  Coefficients that let values grow or that
-// amplify small ones further than 8 iterations of a = 3.4445 do stay in bf16,
-// which has fp32's range.
-inline bool ns_grouped_run(int k, double a, double b, double c) {
+// x h(x^2) and of h, h(t) = a + b t + c t^2.  Coefficients that let values grow or
+// that amplify small ones further than 8 iterations of a = 3.4445 do stay in the
+// iterated form.
+inline bool ns_grouped_run(int k, double a, double b, double c, NsScales* scales = nullptr) {
     if (k < kMinGroupedSteps || k > kMaxGroupedSteps) return false;
     if (!(std::isfinite(a) && std::isfinite(b) && std::isfinite(c))) return false;
     double m = 1.0 + 1.0 / 64, amp = 1.0;       // bound of the singular values; of the gain so far
+    double a_max = 0.0, h_max = 0.0, ha_max = 0.0;   // of A, H and H A over the run
     for (int i = 0; i < k; ++i) {
         // extrema of h on [0, m^2] and of x h(x^2) on [0, m]
         auto h = [&](double t) { return std::fabs(a + b * t + c * t * t); };
@@ -76,13 +96,17 @@ inline bool ns_grouped_run(int k, double a, double b, double c) {
             const double t = -a / (3.0 * b);
             if (t > 0.0 && t < m * m) pmax = std::fmax(pmax, std::sqrt(t) * h(t));
         }
-        // H and Q (a product of up to three H) below 2^12, kScaleA * (H A) and
-        // kScaleX * X below 2^14.
         if (!(hmax <= 16.0) || !(pmax <= 3.0) || !(m * pmax <= 8.0)) return false;
         amp *= hmax;
         if (!(amp <= 32768.0)) return false;
+        a_max = std::fmax(a_max, m * m);
+        h_max = std::fmax(h_max, hmax);
+        ha_max = std::fmax(ha_max, m * pmax);
         m = std::fmax(pmax, 1e-3) * (1.0 + 1.0 / 64);
     }
+    if (scales != nullptr)
+        *scales = {ns_scale_to_fp16(a_max), ns_scale_to_fp16(h_max), ns_scale_to_fp16(ha_max),
+                   ns_scale_to_fp16(h_max * h_max)};
     return true;
 }
 
@@ -103,18 +127,19 @@ inline bool ns_grouped_shape(int64_t p, int64_t q, int64_t tiles) {
 }
 
 // The grouped form's operations; returns their number (at most kMaxGroupedOps).
+// (coefficients that may not take the form: the same products, scales 1)
 inline int ns_grouped_ops(int k, float a, float b, float c, NsOp* ops) {
+    NsScales sc;
+    ns_grouped_run(k, a, b, c, &sc);
     int n = 0;
     for (int kind = kGram; kind <= kBX; ++kind) ops[n++] = ns_iterated_op(0, kind, false, a, b, c);
-    // The first iterate goes out as fp16, scaled.
-    ops[n - 1].out16 = 1;
-    ops[n - 1].gamma = kScaleX;
     int cur = 1;                                  // the iterate that the next group reads
     for (const int* g = kNsGroups[k]; *g > 0; ++g) {
         const bool last = g[1] == 0;
-        auto op = [&](int kind, int x, int y, int out, float gamma) {
+        auto op = [&](int kind, int x, int y, int out, bool f16, bool out16, float gamma) {
             NsOp o = ns_iterated_op(1, kind, false, a, b, c);
-            o.f16 = o.out16 = 1;
+            o.f16 = f16;
+            o.out16 = out16;
             o.a = static_cast<int8_t>(x);
             o.b = static_cast<int8_t>(y);
             o.e = kBufNone;
@@ -123,31 +148,36 @@ inline int ns_grouped_ops(int k, float a, float b, float c, NsOp* ops) {
             o.gamma = gamma;
             ops[n++] = o;
         };
-        op(kGram, kBufX + cur, kBufX + cur, 0, kScaleA / (kScaleX * kScaleX));
+        op(kGram, kBufX + cur, kBufX + cur, 0, false, true, sc.a);
         int q = -1;                               // buffer of the running product Q
+        float q_scale = 1.f;
         for (int j = 0; j < *g; ++j) {
+            const bool end = j + 1 == *g;         // Q is complete: bf16, the type of X
             const int h = q == 1 ? 2 : 1;         // H next to A (buffer 0) and Q
-            op(kPoly, 0, 0, h, c / (kScaleA * kScaleA));
+            const float hs = q < 0 && end ? 1.f : sc.h;
+            op(kPoly, 0, 0, h, true, !(q < 0 && end), hs * c / (sc.a * sc.a));
             ops[n - 1].e = 0;
-            ops[n - 1].alpha = a;
-            ops[n - 1].beta = b / kScaleA;
+            ops[n - 1].alpha = hs * a;
+            ops[n - 1].beta = hs * b / sc.a;
             int free_buf = 6 - h - (q < 0 ? 3 : q);   // buffers 1 .. 3 without h and q
             if (q < 0) {
                 q = h;
+                q_scale = hs;
                 free_buf = h == 1 ? 2 : 1;
             } else {
-                op(kPoly, h, q, free_buf, 1.f);
+                const float s = end ? 1.f : sc.q;
+                op(kPoly, h, q, free_buf, true, !end, s / (sc.h * q_scale));
                 const int old = q;
                 q = free_buf;
+                q_scale = s;
                 free_buf = old;
             }
-            if (j + 1 < *g) {
-                op(kPoly, h, 0, free_buf, 1.f);   // H A
-                op(kPoly, free_buf, h, 0, 1.f);   // (H A) H over A
+            if (!end) {
+                op(kPoly, h, 0, free_buf, true, true, sc.ha / (sc.h * sc.a));   // H A
+                op(kPoly, free_buf, h, 0, true, true, sc.a / (sc.ha * sc.h));   // (H A) H over A
             }
         }
-        op(kBX, q, kBufX + cur, last ? kBufO : kBufX + (cur ^ 1), last ? 1.f / kScaleX : 1.f);
-        if (last) ops[n - 1].out16 = 0;           // O is bf16
+        op(kBX, q, kBufX + cur, last ? kBufO : kBufX + (cur ^ 1), false, false, 1.f);
         cur ^= 1;
     }
     return n;
