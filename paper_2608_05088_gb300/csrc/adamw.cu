@@ -76,7 +76,7 @@ struct AdamBind {
 // double: the update kernel itself does no fp64 arithmetic).
 __global__ void adamw_bind_kernel(const __grid_constant__ AdamBind B, AdamPtrs* __restrict__ table) {
     malt::chain_wait();
-    const int i = threadIdx.x;
+    const int i = malt::after_wait(static_cast<int>(threadIdx.x));
     if (i < B.count) table[B.offset + i] = B.p[i];
     if (i == 0 && B.tcount != nullptr) {
         const long long tc = *B.tcount + 1;                      // 1-based step count
@@ -129,8 +129,9 @@ adamw_kernel(const AdamDesc* __restrict__ desc, const AdamPtrs* __restrict__ ptr
     const int64_t begin = static_cast<int64_t>(blockIdx.x - __ldg(pref + k)) * kAdamChunk;
     const int64_t end = d.numel < begin + kAdamChunk ? d.numel : begin + kAdamChunk;
     // Bias corrections of this step t, computed by the bind launch.
-    const float step = factors[0];
-    const float inv_sqrt_bc2 = factors[1];
+    const float* const f = malt::after_wait(factors);
+    const float step = f[0];
+    const float inv_sqrt_bc2 = f[1];
     const bool gbf = d.g_bf16 != 0;
     const int64_t vec_end = begin + ((end - begin) / kAdamVec) * kAdamVec;
     constexpr int64_t kPass = static_cast<int64_t>(kAdamThreads) * kAdamVec * kAdamInFlight;

@@ -24,11 +24,18 @@ __device__ __forceinline__ void chain_wait() {
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
 }
 
-// The index, opaque to the compiler: a read-only load that it addresses cannot be
-// moved above the wait before it.
+// The index or pointer, opaque to the compiler: an access that it addresses cannot be
+// moved above the wait before it.  The wait alone does not hold back accesses through
+// a __restrict__ pointer, which the compiler may take for memory that nothing else
+// changes: every access through one to what a launch of the chain writes goes by here.
 __device__ __forceinline__ int after_wait(int i) {
     asm volatile("" : "+r"(i)::"memory");
     return i;
+}
+template <typename T>
+__device__ __forceinline__ T* after_wait(T* p) {
+    asm volatile("" : "+l"(p)::"memory");
+    return p;
 }
 
 template <typename... Params, typename... Args>

@@ -1,0 +1,36 @@
+"""Launches that overlap the one before them read what it wrote, never what the
+launch before that did: steps queued back to back, with nothing between them, at
+the start of a run, where every step's factors differ from the last one's by far
+more than the tolerance."""
+import numpy as np
+import pytest
+
+import oracle.adamw_ref as aref
+from tests.test_gpu_whole_optimizer import AdamRun
+
+pytestmark = pytest.mark.gpu
+
+
+def test_adamw_early_steps():
+    """Under a constant gradient every step moves w by lr (m_hat = g, v_hat = g^2).
+    With the factors of the step before, step t would move it by
+    (1 - b1^t) / (1 - b1^(t-1)) sqrt((1 - b2^(t-1)) / (1 - b2^t)) of that: 1.36 at
+    t = 2, 1.01 at t = 20."""
+    run = AdamRun([(5,), (1000,), (70001,)], [0.0, 0.1, 0.0], lr=0.01, seed=75)
+    steps = 20
+    grads = run.draw()
+    for t, g in zip(run.g, grads):
+        t.copy_(run.torch.from_numpy(g))
+    run.torch.cuda.synchronize()
+    for _ in range(steps):
+        run.opt.step(run.hp)
+    for i, g in enumerate(grads):
+        w, wd = run.w0[i].astype(np.float64), float(np.float32(run.wds[i]))
+        for _ in range(steps):
+            w, _ = aref.adamw_step_ref(w, g.astype(np.float64), run.st_ref[i], run.hp_ref, weight_decay=wd)
+        got = run.w[i].double().cpu().numpy()
+        # per step 1e-5 of the step and two ulps of w (tests/test_gpu_whole_optimizer.py)
+        ulp = np.spacing(np.maximum(np.abs(run.w0[i]), np.abs(got)).astype(np.float32))
+        assert np.all(np.abs(got - w) <= steps * (1e-5 * run.lr + 2.0 * ulp)), i
+    assert run.opt.get_step() == steps
+    run.close()
