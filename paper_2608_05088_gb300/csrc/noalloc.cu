@@ -61,7 +61,7 @@ noalloc_stats_kernel(const __grid_constant__ MatDesc d, const __grid_constant__ 
                      float mu1) {
     __shared__ __align__(16) float colsh[8 * malt::kStatCols];
     malt::chain_wait();
-    malt::blk::stats_block<true>(d, up, blockIdx.x, mu1, threadIdx.x, colsh);
+    malt::blk::stats_block<true>(d, up, malt::after_wait(static_cast<int>(blockIdx.x)), mu1, threadIdx.x, colsh);
 }
 
 // EMAs of the statistics and the diagonal preconditioners (Algorithm 1, l_t,
@@ -71,7 +71,7 @@ __global__ void __launch_bounds__(256)
 noalloc_finalize_kernel(const __grid_constant__ MatDesc d, const __grid_constant__ UserPtrs up,
                         float mu2, float eps) {
     malt::chain_wait();
-    const int x = blockIdx.x * blockDim.x + threadIdx.x;
+    const int x = malt::after_wait(static_cast<int>(blockIdx.x * blockDim.x + threadIdx.x));
     if (x < d.m + d.n) malt::blk::finalize_entry(d, up, x, mu2, eps, 0);
 }
 

@@ -6,6 +6,7 @@ import numpy as np
 import pytest
 
 import oracle.adamw_ref as aref
+import paper_2608_05088_gb300.malt as malt
 from tests.test_gpu_whole_optimizer import AdamRun
 
 pytestmark = pytest.mark.gpu
@@ -15,7 +16,7 @@ def test_adamw_early_steps():
     """Under a constant gradient every step moves w by lr (m_hat = g, v_hat = g^2).
     With the factors of the step before, step t would move it by
     (1 - b1^t) / (1 - b1^(t-1)) sqrt((1 - b2^(t-1)) / (1 - b2^t)) of that: 1.36 at
-    t = 2, 1.01 at t = 20."""
+    t = 2, 1.0006 at t = 20."""
     run = AdamRun([(5,), (1000,), (70001,)], [0.0, 0.1, 0.0], lr=0.01, seed=75)
     steps = 20
     grads = run.draw()
@@ -34,3 +35,30 @@ def test_adamw_early_steps():
         assert np.all(np.abs(got - w) <= steps * (1e-5 * run.lr + 2.0 * ulp)), i
     assert run.opt.get_step() == steps
     run.close()
+
+
+def test_noalloc_calls_back_to_back():
+    """Two matrices in turn through the one scratch array, nothing between the calls:
+    bitwise the results of the same calls with the GPU idle before each.  (A finalize
+    that read the partial sums of the call before would see the other matrix's.)"""
+    import torch
+    g = torch.Generator(device="cuda").manual_seed(76)
+
+    def calls(wait):
+        out = []
+        for m, n, scale in ((392, 1000, 1.0), (1280, 776, 1e3)):
+            G = torch.randn(m, n, generator=g, device="cuda").mul_(scale)
+            out.append((G, torch.zeros_like(G), *(torch.zeros(s, device="cuda") for s in (m, n, m, n))))
+        torch.cuda.synchronize()
+        for _ in range(10):
+            for a in out:
+                assert malt.malt_stats_noalloc(*a) == malt.MALT_OK
+                if wait:
+                    torch.cuda.synchronize()
+        torch.cuda.synchronize()
+        return out
+
+    plain = calls(True)
+    g.manual_seed(76)
+    for a, b in zip(plain, calls(False)):
+        assert all(torch.equal(x, y) for x, y in zip(a, b))
