@@ -33,7 +33,7 @@ __device__ __forceinline__ int find_mat(const int32_t* __restrict__ pref, int nm
 // ---------------------------------------------------------------- binding
 __global__ void bind_kernel(const __grid_constant__ BindParams P, UserPtrs* __restrict__ table) {
     chain_wait();
-    const int i = threadIdx.x;
+    const int i = after_wait(static_cast<int>(threadIdx.x));
     if (i < P.count) table[P.offset + i] = P.p[i];
 }
 
@@ -191,7 +191,7 @@ scalars_kernel(const MatDesc* __restrict__ mats, MatScalars* __restrict__ scal,
     __shared__ float red[32];
     chain_wait();
     const int g = after_wait(static_cast<int>(blockIdx.x));
-    blk::scalars_matrix(mats[g], scal + g, clock, hp, threadIdx.x, red);
+    blk::scalars_matrix(mats[g], scal + g, after_wait(clock), hp, threadIdx.x, red);
 }
 
 // ------------------------------------------------------------------ apply
