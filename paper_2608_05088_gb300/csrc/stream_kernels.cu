@@ -132,7 +132,7 @@ finalize_kernel(const MatDesc* __restrict__ mats, const UserPtrs* __restrict__ p
                 StepHyper hp, StepClock* clock, int identity) {
     chain_wait();
     const int32_t x = blockIdx.x * blockDim.x + threadIdx.x;
-    // (the last thread, which has no entry or a row's short sum)
+    // (the last thread: the launch has one thread more than entries at least)
     if (blockIdx.x == gridDim.x - 1 && threadIdx.x == blockDim.x - 1)
         blk::advance_clock(clock, hp.mu1, hp.mu2, hp.eps, hp.malter);
     if (x >= total) return;
@@ -258,8 +258,7 @@ cudaError_t launch_stats(const MatDesc* mats, const UserPtrs* ptrs, const int32_
 cudaError_t launch_finalize(const MatDesc* mats, const UserPtrs* ptrs, const int32_t* pref,
                             int nmat, int32_t total, const StepHyper& hp, StepClock* clock,
                             int identity, cudaStream_t s) {
-    const int blocks = (total + 255) / 256 > 0 ? (total + 255) / 256 : 1;
-    return launch_chained(finalize_kernel, blocks, 256, 0, s, mats, ptrs, pref, nmat, total, hp, clock,
+    return launch_chained(finalize_kernel, total / 256 + 1, 256, 0, s, mats, ptrs, pref, nmat, total, hp, clock,
                           identity);
 }
 
