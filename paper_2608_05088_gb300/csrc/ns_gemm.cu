@@ -744,8 +744,9 @@ ns_gemm_kernel(const __grid_constant__ NsParams P) {
             const bool rok = row < M;
             const int g = job.g >= 0 ? job.g : C.mat_of[w.b];
             const MatDesc& md = P.mats[g];
-            // Persistent launches read what the launch itself wrote (1/||Mt||,
-            // L, R, A) through L2 only.
+            // (1/||Mt||, L and R come from launches before this one, complete since
+            // chain_wait; the persistent instantiation reads them past L1, where a
+            // tile would find nothing of the last one)
             float sc = op.gamma;
             if (op.kx != 0) {
                 const float k = kPersistent ? __ldcg(&P.scal[g].k) : P.scal[g].k;
@@ -776,13 +777,13 @@ ns_gemm_kernel(const __grid_constant__ NsParams P) {
                     // (Newton-Schulz of GPT-2 Small 719 -> 705 us, one 1280 x 5120
                     // and one 5120 x 1280 matrix 327 -> 320).  (Columns past N are
                     // never stored.)
-                    // Phased: A was written by an earlier launch, so the
-                    // read-only path is safe.  Persistent: A is rewritten each
-                    // iteration inside this launch; read through L2 (ordered by
-                    // the acquire of the dependency's counter).
+                    // Through L2 only: A is rewritten within this launch (persistent,
+                    // ordered by the acquire of the dependency's counter) or by a
+                    // launch that this one overlaps (phased, ordered by chain_wait),
+                    // so it is not read-only for the kernel's lifetime.
                     if (rok && col0 + h * 16 < N)
-                        ld_global_32b<kPersistent>(ein + static_cast<size_t>(row) * ns_ld(N) + col0 + h * 16, dst[2 * h],
-                                                   dst[2 * h + 1]);
+                        ld_global_32b(ein + static_cast<size_t>(row) * ns_ld(N) + col0 + h * 16, dst[2 * h],
+                                      dst[2 * h + 1]);
                     else
                         dst[2 * h] = dst[2 * h + 1] = make_uint4(0u, 0u, 0u, 0u);
                 }
@@ -810,6 +811,7 @@ ns_gemm_kernel(const __grid_constant__ NsParams P) {
                         if (lane == 0) raise_timeout(P, abort_flag, kSiteDepLoad + 32, item, seq);
                         break;
                     }
+                    __syncwarp();   // lane 0's acquire holds for the warp's loads
                 }
                 if (nch > 0) load_ein(0, xin);
             }

@@ -152,18 +152,11 @@ __device__ __forceinline__ int4 ld_shared_v4(const void* p) {
     return v;
 }
 
-// One 32-byte load from global memory (32-byte aligned): through L2 only, or on the
-// read-only path.
-template <bool kL2Only>
+// One 32-byte load from global memory (32-byte aligned), through L2 only.
 __device__ __forceinline__ void ld_global_32b(const void* p, uint4& a, uint4& b) {
-    if constexpr (kL2Only)
-        asm volatile("ld.global.cg.v8.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
-                     : "=r"(a.x), "=r"(a.y), "=r"(a.z), "=r"(a.w), "=r"(b.x), "=r"(b.y), "=r"(b.z), "=r"(b.w)
-                     : "l"(p) : "memory");
-    else
-        asm volatile("ld.global.nc.v8.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
-                     : "=r"(a.x), "=r"(a.y), "=r"(a.z), "=r"(a.w), "=r"(b.x), "=r"(b.y), "=r"(b.z), "=r"(b.w)
-                     : "l"(p));
+    asm volatile("ld.global.cg.v8.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
+                 : "=r"(a.x), "=r"(a.y), "=r"(a.z), "=r"(a.w), "=r"(b.x), "=r"(b.y), "=r"(b.z), "=r"(b.w)
+                 : "l"(p) : "memory");
 }
 
 // --------------------------------------------- cross-CTA signals in global memory
