@@ -312,6 +312,10 @@ typedef struct {
 } malt_ns_op_t;
 int malt_ns_plan(int64_t rows, int64_t cols, int32_t n, const malt_hparams_t* hp, malt_ns_op_t* out,
                  int32_t capacity, int32_t* count);
+/* The same for muon_step, whose frames are not preconditioned: the iterates of
+ * merged runs stay in bf16, and runs of 3 iterations are not merged. */
+int malt_muon_ns_plan(int64_t rows, int64_t cols, int32_t n, const malt_hparams_t* hp, malt_ns_op_t* out,
+                      int32_t capacity, int32_t* count);
 
 /* Statistics stage of ONE matrix without any device allocation.
  * The paper has no counterpart: this exists for callers that cannot allocate

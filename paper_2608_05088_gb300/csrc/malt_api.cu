@@ -472,13 +472,14 @@ void build_table(const NsParams& G, const std::vector<int>& slot_class,
 }
 
 // Set a launch group up for a run of k iterations with these coefficients:
-// the classes that can take the grouped form do, when the run may.
-void set_run(NsParams& G, int k, float a, float b, float c, bool grouped) {
+// the classes that can take the grouped form do, when the run may.  raw: frames
+// that are not preconditioned (the same products on other types).
+void set_run(NsParams& G, int k, float a, float b, float c, bool grouped, bool raw) {
     G.ns_steps = k;
     G.a = a;
     G.b = b;
     G.c = c;
-    G.nops = grouped ? ns_grouped_ops(k, a, b, c, G.ops) : 0;
+    G.nops = grouped ? ns_grouped_ops(k, a, b, c, raw, G.ops) : 0;
     for (int j = 0; j < G.nclasses; ++j) G.cls[j].grouped = grouped ? G.cls[j].can_group : 0;
 }
 
@@ -547,14 +548,14 @@ int plan_and_allocate(malt_state* st, const malt_param_t* params, int n) {
         plan_ns_groups(st->classes, n, groups, &slot_class);
         for (size_t gi = 0; gi < groups.size(); ++gi) {
             std::vector<NsEntry> t;
-            set_run(groups[gi], kMaxNsSteps, 0.f, 0.f, 0.f, false);
+            set_run(groups[gi], kMaxNsSteps, 0.f, 0.f, 0.f, false, false);
             build_table(groups[gi], slot_class[gi], st->classes, t);
             st->tables.emplace_back();
             st->tables.back().per_iter = table_per_iter(groups[gi]);
             tables.push_back(std::move(t));
             for (int k = kMinGroupedSteps; k <= kMaxGroupedSteps && any_grouped(groups[gi]); ++k) {
                 t.clear();
-                set_run(groups[gi], k, 0.f, 0.f, 0.f, true);
+                set_run(groups[gi], k, 0.f, 0.f, 0.f, true, false);
                 build_table(groups[gi], slot_class[gi], st->classes, t);
                 st->tables.back().grouped_items[k] = static_cast<int32_t>(t.size());
                 tables.push_back(std::move(t));
@@ -816,15 +817,15 @@ SchedCounters sched_counters(const malt_state* st, const malt_hparams_t* hp) {
 }
 
 // The k Newton-Schulz iterations over every class (after the norms kernel
-// has set 1 / (||Mt|| + ns_eps)).
-int run_newton_schulz(malt_state* st, const malt_hparams_t* hp, cudaStream_t s) {
+// has set 1 / (||Mt|| + ns_eps)).  raw: the frames are not preconditioned (Muon).
+int run_newton_schulz(malt_state* st, const malt_hparams_t* hp, bool raw, cudaStream_t s) {
     thread_local NsParams P;  // ~17 KB of tensor maps: keep off the stack
     const int k = hp->ns_steps;
     const int max_pairs = ns_gemm_max_pairs();
-    const bool grouped_run = ns_grouped_run(k, hp->ns_a, hp->ns_b, hp->ns_c);
+    const bool grouped_run = ns_grouped_run(k, hp->ns_a, hp->ns_b, hp->ns_c, raw);
     auto prepare = [&](const NsParams& G) {
         P = G;
-        set_run(P, k, hp->ns_a, hp->ns_b, hp->ns_c, grouped_run);
+        set_run(P, k, hp->ns_a, hp->ns_b, hp->ns_c, grouped_run, raw);
     };
     bool any_persistent = false;
     for (const NsParams& G : st->ns_groups) any_persistent |= ns_persistent(st, G, max_pairs);
@@ -953,7 +954,7 @@ int run_step(malt_state* st, const malt_param_t* params, int32_t n, const malt_h
         MALT_CUDA(launch_norms(st->d_mats, st->d_scal, nm, hp->ns_eps, malter, sched_counters(st, hp), s),
                   "norms_kernel");
     }
-    rc = run_newton_schulz(st, hp, s);
+    rc = run_newton_schulz(st, hp, muon != 0, s);
     if (rc != MALT_OK) return rc;
     {
         LaunchScope ls(st, MALT_KIND_SCALARS, s);
@@ -1055,6 +1056,33 @@ int run_host_step(malt_state* st, const malt_param_t* params, int32_t n, const m
     }
     MALT_CUDA(cudaEventRecord(st->ev_d2h, st->d2h), "cudaEventRecord(d2h)");
     st->pipe_primed = true;
+    return MALT_OK;
+}
+
+// malt_ns_plan and malt_muon_ns_plan.
+int ns_plan_of_step(int64_t rows, int64_t cols, int32_t n, const malt_hparams_t* hp, bool raw, malt_ns_op_t* out,
+                    int32_t capacity, int32_t* count) {
+    if (count == nullptr || n < 1 || capacity < 0 || (capacity > 0 && out == nullptr)) return MALT_ERR_INVALID_ARG;
+    const int rc = validate_hparams(hp);
+    if (rc != MALT_OK) return rc;
+    malt_param_t p{};
+    p.rows = rows;
+    p.cols = cols;
+    if (rows <= 0 || cols <= 0 || round8(rows) * round8(cols) >= (int64_t{1} << 31)) return MALT_ERR_UNSUPPORTED;
+    std::vector<MatDesc> hmats;
+    std::vector<ShapeClass> classes;
+    const std::vector<malt_param_t> set(static_cast<size_t>(n), p);
+    build_classes(set.data(), n, true, hmats, classes);
+    std::vector<NsParams> groups;
+    plan_ns_groups(classes, n, groups);
+    NsParams& G = groups[0];
+    set_run(G, hp->ns_steps, hp->ns_a, hp->ns_b, hp->ns_c,
+            ns_grouped_run(hp->ns_steps, hp->ns_a, hp->ns_b, hp->ns_c, raw), raw);
+    *count = ns_num_stages(G, G.cls[0]);
+    for (int s = 0; s < std::min(capacity, *count); ++s) {
+        const NsOp o = ns_op(G, G.cls[0], s);
+        out[s] = malt_ns_op_t{o.kind, o.f16, o.out16, o.a, o.b, o.e, o.out, o.kx, o.alpha, o.beta, o.gamma};
+    }
     return MALT_OK;
 }
 
@@ -1325,7 +1353,7 @@ int malt_ns_schedule(const malt_param_t* params, int32_t n, int32_t ns_steps, in
     std::vector<NsEntry> table;
     for (size_t gi = 0; gi < groups.size(); ++gi) {
         NsParams& G = groups[gi];
-        set_run(G, ns_steps, 0.f, 0.f, 0.f, false);
+        set_run(G, ns_steps, 0.f, 0.f, 0.f, false, false);
         build_table(G, slot_class[gi], classes, table);
         for (const NsEntry& e : table) {
             if (total < capacity) {
@@ -1350,27 +1378,12 @@ int malt_ns_schedule(const malt_param_t* params, int32_t n, int32_t ns_steps, in
 
 int malt_ns_plan(int64_t rows, int64_t cols, int32_t n, const malt_hparams_t* hp, malt_ns_op_t* out,
                  int32_t capacity, int32_t* count) {
-    if (count == nullptr || n < 1 || capacity < 0 || (capacity > 0 && out == nullptr)) return MALT_ERR_INVALID_ARG;
-    const int rc = validate_hparams(hp);
-    if (rc != MALT_OK) return rc;
-    malt_param_t p{};
-    p.rows = rows;
-    p.cols = cols;
-    if (rows <= 0 || cols <= 0 || round8(rows) * round8(cols) >= (int64_t{1} << 31)) return MALT_ERR_UNSUPPORTED;
-    std::vector<MatDesc> hmats;
-    std::vector<ShapeClass> classes;
-    const std::vector<malt_param_t> set(static_cast<size_t>(n), p);
-    build_classes(set.data(), n, true, hmats, classes);
-    std::vector<NsParams> groups;
-    plan_ns_groups(classes, n, groups);
-    NsParams& G = groups[0];
-    set_run(G, hp->ns_steps, hp->ns_a, hp->ns_b, hp->ns_c, ns_grouped_run(hp->ns_steps, hp->ns_a, hp->ns_b, hp->ns_c));
-    *count = ns_num_stages(G, G.cls[0]);
-    for (int s = 0; s < std::min(capacity, *count); ++s) {
-        const NsOp o = ns_op(G, G.cls[0], s);
-        out[s] = malt_ns_op_t{o.kind, o.f16, o.out16, o.a, o.b, o.e, o.out, o.kx, o.alpha, o.beta, o.gamma};
-    }
-    return MALT_OK;
+    return ns_plan_of_step(rows, cols, n, hp, false, out, capacity, count);
+}
+
+int malt_muon_ns_plan(int64_t rows, int64_t cols, int32_t n, const malt_hparams_t* hp, malt_ns_op_t* out,
+                      int32_t capacity, int32_t* count) {
+    return ns_plan_of_step(rows, cols, n, hp, true, out, capacity, count);
 }
 
 const char* malt_status_string(int code) {

@@ -14,31 +14,35 @@
 //    symmetric themselves, and every one is computed as an upper triangle.
 //    With q = 4 p a merged iteration costs 4 p^3 in place of 13 p^3.
 //
-// Rounding.  X stays in bf16 in both forms: its rows and columns may differ by many
-// decades (a frame that is not preconditioned, rows without gradients), and bf16 has
-// fp32's range.  With X in fp16, whatever its scale, a column 1e-10 of the others
-// left with an error of 1.  The p x p matrices of a group are fp16, 11 significant
-// bits in place of 8: in bf16 the grouped form loses accuracy, since A carries the
-// squared singular values (1.5 times the iterated form's error, 2 in the worst row).
-// Their entries are bounded (|p(x)| stays near 1), so each is stored times the
-// power of two that puts its bound at 2^15 (ns_grouped_run): an entry of A keeps
-// all its bits down to 2^-28 of a unit singular value squared, one of H down to
-// 2^-27.  What is left of the range: the entries that couple a small row of X with the
-// others are that small where the row is below 1e-8 of the frame.  With half the rows
-// scaled by 1e-8 nothing is lost (0.004 - 0.011 in those rows, iterated 0.009 - 0.018);
-// by 1e-9 it is 0.005 - 0.08, by 1e-10 0.007 - 0.7, by 1e-12 they keep only the leading
-// factor a^k.  The running product that is applied to X goes out in bf16, X's type.
+// Rounding.  In bf16 the grouped form loses accuracy, since A carries the squared
+// singular values (1.5 times the iterated form's error, 2 in the worst row), so the
+// p x p matrices of a group are fp16: 11 significant bits in place of 8.  Their
+// entries are bounded (|p(x)| stays near 1), so each is stored times the power of two
+// that brings its bound near fp16's largest value (ns_grouped_run): A and H A times
+// 2^14, H times 2^13 with the default coefficients.  The iterates X are
+//  * fp16 times 2^15 for preconditioned frames (MALT, MALTER: L M R, whose rows and
+//    columns are drawn together);
+//  * bf16, which has fp32's range, for frames as they are (Muon).  A column 1e-10 of
+//    the others leaves fp16 with an error of 1 at any scale.  The running product that
+//    is applied to X goes out in X's type; bf16 costs it accuracy, and at k = 3 the
+//    worst column gets 1.0 - 1.3 times the iterated form's error, so these runs stay
+//    iterated.
+// The first iteration keeps bf16, because Mt's scale is not known before it.
 //
-// Against fp64, k = 4 to 8, relative to the iterated form's error on frames with
-// log-normal scales (sigma 0 to 3, as they are and preconditioned): the whole frame
-// 0.6 - 0.9, the median row and column 0.5 - 0.9, the worst row and column 0.4 - 0.95
-// (geometric means over shapes 64 x 128 to 512 x 2048).  At k = 3 the worst column is
-// 1.0 - 1.3, so 3 iterations stay iterated.  tests/test_ns_plan.py reads the plan from
-// the library and runs its arithmetic on the CPU, on these frames and on geometric,
-// low-rank, graded and blocked ones.
+// Error against fp64 in terms of the iterated form's, on frames with log-normal scales
+// of sigma 0 to 3 (geometric means over 64 x 128 to 512 x 2048, k = 3 to 8): preconditioned,
+// fp16, the whole frame 0.3 - 0.65, the worst row and column 0.2 - 0.7; as they are,
+// bf16, 0.6 - 0.9 and 0.5 - 0.95.  Rows and columns far smaller than the rest: half
+// of them 1e-8 of the others have errors of 0.005 - 0.015 (iterated 0.01 - 0.03; k = 3:
+// the same down to 1e-7).  Below that the range of fp16 ends: at 1e-9 0.03 - 0.14, at 1e-10
+// 0.3 - 1; with X in bf16 columns have no such limit and rows 0.005 - 0.08 at 1e-9.
+// An update that small against the others moves W by less than W's own fp32 rounding.
+// tests/test_ns_plan.py reads the plan from the library and runs its arithmetic on
+// the CPU, on these frames and on geometric, low-rank, graded and blocked ones.
 //
 // Which form runs (ns_grouped_run, ns_grouped_shape) follows from k, from the
-// coefficients, from the shape and from the size of the set.
+// coefficients, from whether the frames are preconditioned, from the shape and from
+// the size of the set.
 #pragma once
 #include <cmath>
 #include <cstdint>
@@ -47,36 +51,37 @@
 
 namespace malt {
 
-// Groups of a k-iteration run after the first iteration (k = 4 .. 8), zero
+// Groups of a k-iteration run after the first iteration (k = 3 .. 8), zero
 // ended.  Pairs; three at a time loses accuracy on ill-conditioned frames, so
 // it is taken only where it ends the longest run.
-constexpr int kMinGroupedSteps = 4, kMaxGroupedSteps = 8;
+constexpr int kMinGroupedSteps = 3, kMinGroupedStepsRaw = 4, kMaxGroupedSteps = 8;
 constexpr int kNsGroups[kMaxGroupedSteps + 1][4] = {
-    {0}, {0}, {0}, {0}, {2, 1, 0}, {2, 2, 0}, {2, 2, 1, 0}, {2, 2, 2, 0}, {2, 2, 3, 0}};
+    {0}, {0}, {0}, {2, 0}, {2, 1, 0}, {2, 2, 0}, {2, 2, 1, 0}, {2, 2, 2, 0}, {2, 2, 3, 0}};
 
-// Factors (powers of two) by which a group's fp16 matrices are stored.
+// Factors (powers of two) by which the fp16 matrices are stored: X, A, H A, and the
+// product of 1, 2 or 3 H.
 struct NsScales {
-    float a = 1.f, h = 1.f, ha = 1.f, q = 1.f;   // A, H, H A, and a running product that grows further
+    float x = 1.f, a = 1.f, ha = 1.f, h[3] = {1.f, 1.f, 1.f};
 };
 
-// The power of two that brings a bound to at most 2^15, half of fp16's largest
-// value: rounding moves what the bounds say by a few percent at most.
+// The largest power of two that keeps a bound below 2^15.5, 0.7 of fp16's largest
+// value: the bounds have 1/64 to spare per iteration, rounding moves values by less.
 inline float ns_scale_to_fp16(double bound) {
-    return static_cast<float>(std::exp2(std::floor(15.0 - std::log2(std::fmax(bound, 1.0)))));
+    return static_cast<float>(std::exp2(std::floor(15.5 - std::log2(std::fmax(bound, 1.0)))));
 }
 
 // Whether a run of k iterations with these coefficients may take the grouped
-// form, and its scales: the fp16 values must stay in range.  The
-// singular values of the first iterate are at most 1 (X is divided by its
-// Frobenius norm), so the range of every later one follows from the extrema of
-// x h(x^2) and of h, h(t) = a + b t + c t^2.  Coefficients that let values grow or
+// form (raw: on frames that are not preconditioned), and its scales: the fp16
+// values must stay in range.  The singular values of the first iterate are at most
+// 1 (X is divided by its Frobenius norm), so the range of every later one follows
+// from the extrema of x h(x^2) and of h, h(t) = a + b t + c t^2.  Coefficients that let values grow or
 // that amplify small ones further than 8 iterations of a = 3.4445 do stay in the
 // iterated form.
-inline bool ns_grouped_run(int k, double a, double b, double c, NsScales* scales = nullptr) {
-    if (k < kMinGroupedSteps || k > kMaxGroupedSteps) return false;
+inline bool ns_grouped_run(int k, double a, double b, double c, bool raw, NsScales* scales = nullptr) {
+    if (k < (raw ? kMinGroupedStepsRaw : kMinGroupedSteps) || k > kMaxGroupedSteps) return false;
     if (!(std::isfinite(a) && std::isfinite(b) && std::isfinite(c))) return false;
     double m = 1.0 + 1.0 / 64, amp = 1.0;       // bound of the singular values; of the gain so far
-    double a_max = 0.0, h_max = 0.0, ha_max = 0.0;   // of A, H and H A over the run
+    double x_max = 0.0, a_max = 0.0, h_max = 0.0, ha_max = 0.0;   // of X (once iterated), A, H and H A
     for (int i = 0; i < k; ++i) {
         // extrema of h on [0, m^2] and of x h(x^2) on [0, m]
         auto h = [&](double t) { return std::fabs(a + b * t + c * t * t); };
@@ -102,11 +107,13 @@ inline bool ns_grouped_run(int k, double a, double b, double c, NsScales* scales
         a_max = std::fmax(a_max, m * m);
         h_max = std::fmax(h_max, hmax);
         ha_max = std::fmax(ha_max, m * pmax);
+        x_max = std::fmax(x_max, pmax * (1.0 + 1.0 / 64));
         m = std::fmax(pmax, 1e-3) * (1.0 + 1.0 / 64);
     }
     if (scales != nullptr)
-        *scales = {ns_scale_to_fp16(a_max), ns_scale_to_fp16(h_max), ns_scale_to_fp16(ha_max),
-                   ns_scale_to_fp16(h_max * h_max)};
+        *scales = {ns_scale_to_fp16(x_max), ns_scale_to_fp16(a_max), ns_scale_to_fp16(ha_max),
+                   {ns_scale_to_fp16(h_max), ns_scale_to_fp16(h_max * h_max),
+                    ns_scale_to_fp16(h_max * h_max * h_max)}};
     return true;
 }
 
@@ -127,12 +134,16 @@ inline bool ns_grouped_shape(int64_t p, int64_t q, int64_t tiles) {
 }
 
 // The grouped form's operations; returns their number (at most kMaxGroupedOps).
-// (coefficients that may not take the form: the same products, scales 1)
-inline int ns_grouped_ops(int k, float a, float b, float c, NsOp* ops) {
+// (a run that may not take the form: the same products, scales 1)
+inline int ns_grouped_ops(int k, float a, float b, float c, bool raw, NsOp* ops) {
     NsScales sc;
-    ns_grouped_run(k, a, b, c, &sc);
+    ns_grouped_run(k, a, b, c, raw, &sc);
+    const bool x16 = !raw;
+    const float xs = x16 ? sc.x : 1.f;
     int n = 0;
     for (int kind = kGram; kind <= kBX; ++kind) ops[n++] = ns_iterated_op(0, kind, false, a, b, c);
+    ops[n - 1].out16 = x16;
+    ops[n - 1].gamma = xs;
     int cur = 1;                                  // the iterate that the next group reads
     for (const int* g = kNsGroups[k]; *g > 0; ++g) {
         const bool last = g[1] == 0;
@@ -148,36 +159,38 @@ inline int ns_grouped_ops(int k, float a, float b, float c, NsOp* ops) {
             o.gamma = gamma;
             ops[n++] = o;
         };
-        op(kGram, kBufX + cur, kBufX + cur, 0, false, true, sc.a);
+        op(kGram, kBufX + cur, kBufX + cur, 0, x16, true, sc.a / (xs * xs));
         int q = -1;                               // buffer of the running product Q
         float q_scale = 1.f;
         for (int j = 0; j < *g; ++j) {
-            const bool end = j + 1 == *g;         // Q is complete: bf16, the type of X
+            const bool end = j + 1 == *g;         // Q is complete: X's type
+            const bool to16 = !end || x16;
+            const float s = to16 ? sc.h[j] : 1.f;    // of Q
             const int h = q == 1 ? 2 : 1;         // H next to A (buffer 0) and Q
-            const float hs = q < 0 && end ? 1.f : sc.h;
-            op(kPoly, 0, 0, h, true, !(q < 0 && end), hs * c / (sc.a * sc.a));
+            const float hs = q < 0 ? s : sc.h[0];
+            op(kPoly, 0, 0, h, true, q >= 0 || to16, hs * c / (sc.a * sc.a));
             ops[n - 1].e = 0;
             ops[n - 1].alpha = hs * a;
             ops[n - 1].beta = hs * b / sc.a;
             int free_buf = 6 - h - (q < 0 ? 3 : q);   // buffers 1 .. 3 without h and q
             if (q < 0) {
                 q = h;
-                q_scale = hs;
                 free_buf = h == 1 ? 2 : 1;
             } else {
-                const float s = end ? 1.f : sc.q;
-                op(kPoly, h, q, free_buf, true, !end, s / (sc.h * q_scale));
+                op(kPoly, h, q, free_buf, true, to16, s / (hs * q_scale));
                 const int old = q;
                 q = free_buf;
-                q_scale = s;
                 free_buf = old;
             }
+            q_scale = s;
             if (!end) {
-                op(kPoly, h, 0, free_buf, true, true, sc.ha / (sc.h * sc.a));   // H A
-                op(kPoly, free_buf, h, 0, true, true, sc.a / (sc.ha * sc.h));   // (H A) H over A
+                op(kPoly, h, 0, free_buf, true, true, sc.ha / (hs * sc.a));   // H A
+                op(kPoly, free_buf, h, 0, true, true, sc.a / (sc.ha * hs));   // (H A) H over A
             }
         }
-        op(kBX, q, kBufX + cur, last ? kBufO : kBufX + (cur ^ 1), false, false, 1.f);
+        // (O is bf16)
+        op(kBX, q, kBufX + cur, last ? kBufO : kBufX + (cur ^ 1), x16, x16 && !last,
+           1.f / (last ? q_scale * xs : q_scale));
         cur ^= 1;
     }
     return n;

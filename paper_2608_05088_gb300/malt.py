@@ -39,7 +39,7 @@ EXPORTS = ("malt_init_state", "malt_step", "malter_step", "malt_get_scalars",
            "malt_ns_schedule", "malt_debug_timeout_site", "malt_debug_precond",
            "malt_set_weight_copies", "malt_adamw_init_state", "malt_adamw_step",
            "malt_adamw_get_step", "malt_adamw_set_step", "malt_adamw_destroy_state",
-           "malt_debug_check_guards", "malt_ns_plan")
+           "malt_debug_check_guards", "malt_ns_plan", "malt_muon_ns_plan")
 NOALLOC_SCRATCH_FLOATS = 1048576
 KIND_NAMES = ("bind", "stats", "finalize", "prescale", "norms", "ns_gram", "ns_poly", "ns_bx",
               "scalars", "apply", "ns_persistent", "pad")
@@ -155,8 +155,9 @@ def load(build_if_missing: bool = False) -> ctypes.CDLL:
     lib.malt_adamw_destroy_state.argtypes = [vp]
     lib.malt_adamw_destroy_state.restype = None
     lib.malt_ns_schedule.restype = ctypes.c_int
-    lib.malt_ns_plan.argtypes = [i64, i64, i32, P(malt_hparams_t), P(malt_ns_op_t), i32, P(i32)]
-    lib.malt_ns_plan.restype = ctypes.c_int
+    for name in ("malt_ns_plan", "malt_muon_ns_plan"):
+        getattr(lib, name).argtypes = [i64, i64, i32, P(malt_hparams_t), P(malt_ns_op_t), i32, P(i32)]
+        getattr(lib, name).restype = ctypes.c_int
     for name in ("malt_init_state", "malt_step", "malter_step", "malt_get_scalars",
                  "malt_set_scalars", "malt_check", "malt_debug_direction",
                  "malt_debug_scalars", "malt_debug_wait_timeout", "malt_profile_enable",
@@ -475,12 +476,13 @@ def malt_ns_schedule(shapes, ns_steps: int):
     return out
 
 
-def malt_ns_plan(rows: int, cols: int, n: int, hp: malt_hparams_t):
-    """The products a step runs on each matrix of a set of n rows x cols
-    matrices (malt_ns_op_t list; host only, no GPU)."""
+def malt_ns_plan(rows: int, cols: int, n: int, hp: malt_hparams_t, muon: bool = False):
+    """The products a step (a Muon step) runs on each matrix of a set of n rows x
+    cols matrices (malt_ns_op_t list; host only, no GPU)."""
     ops = (malt_ns_op_t * 192)()
     count = ctypes.c_int32(0)
-    _check(load().malt_ns_plan(rows, cols, n, ctypes.byref(hp), ops, len(ops), ctypes.byref(count)), "malt_ns_plan")
+    name = "malt_muon_ns_plan" if muon else "malt_ns_plan"
+    _check(getattr(load(), name)(rows, cols, n, ctypes.byref(hp), ops, len(ops), ctypes.byref(count)), name)
     return list(ops[:count.value])
 
 

@@ -3,7 +3,8 @@
 stored matrices, fp32 products, symmetric products mirrored from their upper
 triangle.
 
-The grouped form (wide frames, 4 to 8 iterations) must compute the oracle's
+The grouped form (wide frames, 3 to 8 iterations, 4 to 8 where the frames are not
+preconditioned: Muon) must compute the oracle's
 iteration and be no further from fp64 than the iterated bf16 form that it
 replaces: as a whole frame, and row by row and column by column, so that rows
 and columns far smaller than the rest keep their relative accuracy too.
@@ -82,11 +83,14 @@ def is_grouped(ops):
     return any(o.in_f16 for o in ops)
 
 
-@pytest.mark.parametrize("k", [4, 5, 6, 7, 8])
-def test_grouped_form(malt, k):
+GROUPED = [(k, False) for k in range(3, 9)] + [(k, True) for k in range(4, 9)]
+
+
+@pytest.mark.parametrize("k,muon", GROUPED)
+def test_grouped_form(malt, k, muon):
     hp = malt.hparams(ns_steps=k)
     for p, q in ((64, 512), (128, 256)):
-        ops = malt.malt_ns_plan(p, q, 1000, hp)
+        ops = malt.malt_ns_plan(p, q, 1000, hp, muon)
         assert is_grouped(ops)
         for name, Mt in frames(p, q):
             Mt = Mt.astype(np.float32).astype(np.float64)
@@ -98,31 +102,33 @@ def test_grouped_form(malt, k):
             assert err < 1.1 * old, (p, q, name, err, old)
 
 
-def graded_frames(p, q):
-    """Rows or columns far smaller than the rest, and scales of sigma 3 as they are
-    (Muon's frames) and preconditioned."""
+def graded_frames(p, q, muon, k):
+    """Rows or columns far smaller than the rest, down to where the form's range ends,
+    and scales of sigma 3, preconditioned or (Muon) as they are."""
     rng = np.random.default_rng(11)
     X, i, j = rng.standard_normal((p, q)), np.arange(p), np.arange(q)
-    for e in (4, 6, 8):
+    for e in (4, 6) if k == 3 else (4, 6, 8):
         yield f"half the rows 1e-{e}", X * np.where(i < p // 2, 1.0, 10.0 ** -e)[:, None]
-    for e in (6, 10, 14):
+    for e in (6, 10, 14) if muon else (6, 7) if k == 3 else (6, 8):
         yield f"half the columns 1e-{e}", X * np.where(j < q // 2, 1.0, 10.0 ** -e)[None, :]
     B = X * ((i < p // 2)[:, None] == (j < q // 2)[None, :])
     yield "two blocks, one 1e-6", B * np.where(i < p // 2, 1.0, 1e-6)[:, None]
     yield "all 1e-12 (below ns_eps)", X * 1e-12
     G = X * np.exp(3.0 * rng.standard_normal(p))[:, None] * np.exp(3.0 * rng.standard_normal(q))[None, :]
-    yield "sigma 3", G
-    L, R = ((G * G).sum(1) * 0.01 + 1e-8) ** -0.125, ((G * G).sum(0) * 0.01 + 1e-8) ** -0.125
-    yield "sigma 3, preconditioned", L[:, None] * G * R[None, :]
+    if muon:
+        yield "sigma 3", G
+    else:
+        L, R = ((G * G).sum(1) * 0.01 + 1e-8) ** -0.125, ((G * G).sum(0) * 0.01 + 1e-8) ** -0.125
+        yield "sigma 3, preconditioned", L[:, None] * G * R[None, :]
 
 
-@pytest.mark.parametrize("k", [4, 5, 6, 7, 8])
-def test_grouped_form_by_rows_and_columns(malt, k):
+@pytest.mark.parametrize("k,muon", GROUPED)
+def test_grouped_form_by_rows_and_columns(malt, k, muon):
     hp = malt.hparams(ns_steps=k)
     for p, q in ((128, 512), (256, 1024)):
-        ops = malt.malt_ns_plan(p, q, 1000, hp)
+        ops = malt.malt_ns_plan(p, q, 1000, hp, muon)
         assert is_grouped(ops)
-        for name, Mt in graded_frames(p, q):
+        for name, Mt in graded_frames(p, q, muon, k):
             Mt = Mt.astype(np.float32).astype(np.float64)
             want = ref.newton_schulz(Mt, k, tuple(float(np.float32(c)) for c in ref.DEFAULT_NS_COEFFS))
             new, old = run_plan(ops, Mt) - want, newton_schulz_bf16(Mt, k) - want
@@ -137,6 +143,29 @@ def test_grouped_form_by_rows_and_columns(malt, k):
                 assert e_new.max() < 2.0 * e_old.max(), (p, q, name, axis, e_new.max(), e_old.max())
 
 
+def test_values_stay_in_range(malt):
+    """No stored value of a grouped run reaches fp16's largest, for the frames whose
+    iterates are largest (constant singular values at the maximum of the polynomial)
+    and for the coefficients with the widest bounds that the rule admits."""
+    rng = np.random.default_rng(5)
+    p, q = 64, 128
+    U = np.linalg.qr(rng.standard_normal((p, p)))[0]
+    V = np.linalg.qr(rng.standard_normal((q, p)))[0].T
+    for co in (ref.DEFAULT_NS_COEFFS, (1.5, -0.5, 0.0), (4.0848, -6.8946, 2.9270), (4.5, -2.88, 0.3686)):
+        for k in range(3, 9):
+            for muon in (False, True):
+                ops = malt.malt_ns_plan(p, q, 1000, malt.hparams(ns_steps=k, ns_coeffs=co), muon)
+                if not is_grouped(ops):
+                    continue
+                for r in (1, 2, 3, 4, 8, 20, p):
+                    s = np.where(np.arange(p) < r, 1.0, 1e-3)
+                    # rank r: singular values 1 / sqrt(r); a single entry; a single row
+                    for Mt in ((U * s) @ V, np.eye(p, q) * s[:, None], np.where(np.arange(p) < r, 1.0, 0.0)[:, None]
+                               * np.ones((1, q))):
+                        out = run_plan(ops, Mt.astype(np.float32).astype(np.float64))
+                        assert np.all(np.isfinite(out)), (co, k, muon, r)
+
+
 def test_rule(malt):
     hp = malt.hparams
     default = hp()
@@ -145,8 +174,8 @@ def test_rule(malt):
         assert is_grouped(malt.malt_ns_plan(*shape, n, default)), shape
     for shape, n in (((1024, 2040), 100), ((4096, 4096), 1), ((256, 512), 1), ((512, 1024), 32), ((768, 768), 12)):
         assert not is_grouped(malt.malt_ns_plan(*shape, n, default)), shape
-    for k in (1, 2, 3, 9, 64):
-        ops = malt.malt_ns_plan(256, 1024, 500, hp(ns_steps=k))
+    for k, muon in ((1, False), (2, False), (3, True), (9, False), (64, True)):
+        ops = malt.malt_ns_plan(256, 1024, 500, hp(ns_steps=k), muon)
         assert not is_grouped(ops) and len(ops) == 3 * k
     # the classical cubic is in range; growing or strongly amplifying runs are not
     assert is_grouped(malt.malt_ns_plan(256, 1024, 500, hp(ns_coeffs=(1.5, -0.5, 0.0))))
