@@ -312,6 +312,12 @@ static_assert(kMaxStages >= kMaxGroupedOps, "one row of counters per stage");
 constexpr int kAutoPersistentWaves = 16;
 constexpr int kStatusWords = 8;
 
+// 256 x 256 tiles of a symmetric p x p product.
+int64_t wide_sym_tiles(int64_t p) {
+    const int64_t tp = (p + kTileM - 1) / kTileM;
+    return tp * (tp + 1) / 2;
+}
+
 // Per-matrix descriptions and shape classes (one per NS frame p x q, in order
 // of first appearance).  Host only.
 //
@@ -362,10 +368,7 @@ void build_classes(const malt_param_t* params, int n, bool narrow_tiles, std::ve
         d.pre_tc = (c + kPreCols - 1) / kPreCols;
     }
     int64_t tiles = 0;                 // of one symmetric product over the set
-    for (const ShapeClass& C : classes) {
-        const int64_t tp = (C.p + kTileM - 1) / kTileM;
-        tiles += tp * (tp + 1) / 2 * C.batch;
-    }
+    for (const ShapeClass& C : classes) tiles += wide_sym_tiles(C.p) * C.batch;
     int64_t bx_tiles = 0;              // of B*X
     for (const ShapeClass& C : classes)
         bx_tiles += static_cast<int64_t>((C.p + kTileM - 1) / kTileM) * ((C.q + kWideN - 1) / kWideN) * C.batch;
@@ -1065,22 +1068,21 @@ int ns_plan_of_step(int64_t rows, int64_t cols, int32_t n, const malt_hparams_t*
     if (count == nullptr || n < 1 || capacity < 0 || (capacity > 0 && out == nullptr)) return MALT_ERR_INVALID_ARG;
     const int rc = validate_hparams(hp);
     if (rc != MALT_OK) return rc;
-    malt_param_t p{};
-    p.rows = rows;
-    p.cols = cols;
     if (rows <= 0 || cols <= 0 || round8(rows) * round8(cols) >= (int64_t{1} << 31)) return MALT_ERR_UNSUPPORTED;
-    std::vector<MatDesc> hmats;
-    std::vector<ShapeClass> classes;
-    const std::vector<malt_param_t> set(static_cast<size_t>(n), p);
-    build_classes(set.data(), n, true, hmats, classes);
-    std::vector<NsParams> groups;
-    plan_ns_groups(classes, n, groups);
-    NsParams& G = groups[0];
+    // What build_classes and set_run settle for such a set, whatever its size n.
+    NsParams G;
+    std::memset(&G, 0, sizeof(G));
+    G.nclasses = 1;
+    NsClass& C = G.cls[0];
+    const int64_t m = round8(rows), c = round8(cols);
+    C.p = static_cast<int32_t>(std::min(m, c));
+    C.q = static_cast<int32_t>(std::max(m, c));
+    C.can_group = ns_grouped_shape(C.p, C.q, wide_sym_tiles(C.p) * n);
     set_run(G, hp->ns_steps, hp->ns_a, hp->ns_b, hp->ns_c,
             ns_grouped_run(hp->ns_steps, hp->ns_a, hp->ns_b, hp->ns_c, raw), raw);
-    *count = ns_num_stages(G, G.cls[0]);
+    *count = ns_num_stages(G, C);
     for (int s = 0; s < std::min(capacity, *count); ++s) {
-        const NsOp o = ns_op(G, G.cls[0], s);
+        const NsOp o = ns_op(G, C, s);
         out[s] = malt_ns_op_t{o.kind, o.f16, o.out16, o.a, o.b, o.e, o.out, o.kx, o.alpha, o.beta, o.gamma};
     }
     return MALT_OK;

@@ -190,3 +190,14 @@ def test_iterated_form_is_unchanged(malt):
     want = ref.newton_schulz(Mt)
     err, old = _rel(run_plan(malt.malt_ns_plan(96, 96, 1, malt.hparams()), Mt), want), _rel(newton_schulz_bf16(Mt), want)
     assert 0.8 * old < err < 1.25 * old, (err, old)
+
+
+def test_plan_of_any_number_of_matrices(malt):
+    """The plan depends on the set's size through its number of tiles only, and takes
+    no memory in it: a set larger than any memory is answered, not aborted on."""
+    hp = malt.hparams()
+    for shape in ((8, 16), (1280, 5120), (300, 77)):
+        for muon in (False, True):
+            big = malt.malt_ns_plan(*shape, 2 ** 31 - 1, hp, muon)
+            assert is_grouped(big) == (max(shape) >= 2 * min(shape))
+            assert len(malt.malt_ns_plan(*shape, 100000, hp, muon)) == len(big)
