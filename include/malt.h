@@ -292,6 +292,17 @@ int malt_set_ns_schedule(malt_state_t* st, int32_t schedule);
 int malt_ns_schedule(const malt_param_t* params, int32_t n, int32_t ns_steps, int32_t* out,
                      int64_t capacity, int64_t* count);
 
+/* Host only: the work tables that the persistent launches of a step of these
+ * parameters claim from (muon: of a muon_step), entry by entry as they run: with
+ * merged iterations and narrow tiles where the set takes them.  11 int32 per item:
+ * the eight of malt_ns_schedule (kind 1 is any product of two symmetric p x p
+ * matrices, stage s the s-th product of the item's matrix), then the width of the
+ * tile, the class slot and the batch slot.  Only rows and cols of params are read.
+ * Writes min(capacity, total) items and the total to *count; errors as
+ * malt_ns_plan. */
+int malt_ns_tables(const malt_param_t* params, int32_t n, const malt_hparams_t* hp, int32_t muon, int32_t* out,
+                   int64_t capacity, int64_t* count);
+
 /* Host only: the products that a step runs on each matrix of a set of n
  * rows x cols matrices, in order.
  * An operation is out = gamma k^kx (a b) + beta e + alpha I with

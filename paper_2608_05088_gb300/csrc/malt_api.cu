@@ -486,6 +486,16 @@ void set_run(NsParams& G, int k, float a, float b, float c, bool grouped, bool r
     for (int j = 0; j < G.nclasses; ++j) G.cls[j].grouped = grouped ? G.cls[j].can_group : 0;
 }
 
+// The table of a launch group for runs of k iterations in the grouped form, or
+// (grouped false) for kMaxNsSteps iterations of the iterated form, of which a run of
+// k claims the first k table_per_iter(G) entries.  It does not depend on the
+// coefficients or types.
+void run_table(NsParams& G, const std::vector<int>& slot_class, const std::vector<ShapeClass>& classes,
+               int k, bool grouped, std::vector<NsEntry>& out) {
+    set_run(G, grouped ? k : kMaxNsSteps, 0.f, 0.f, 0.f, grouped, false);
+    build_table(G, slot_class, classes, out);
+}
+
 bool any_grouped(const NsParams& G) {
     for (int c = 0; c < G.nclasses; ++c)
         if (G.cls[c].can_group) return true;
@@ -551,15 +561,13 @@ int plan_and_allocate(malt_state* st, const malt_param_t* params, int n) {
         plan_ns_groups(st->classes, n, groups, &slot_class);
         for (size_t gi = 0; gi < groups.size(); ++gi) {
             std::vector<NsEntry> t;
-            set_run(groups[gi], kMaxNsSteps, 0.f, 0.f, 0.f, false, false);
-            build_table(groups[gi], slot_class[gi], st->classes, t);
+            run_table(groups[gi], slot_class[gi], st->classes, kMaxNsSteps, false, t);
             st->tables.emplace_back();
             st->tables.back().per_iter = table_per_iter(groups[gi]);
             tables.push_back(std::move(t));
             for (int k = kMinGroupedSteps; k <= kMaxGroupedSteps && any_grouped(groups[gi]); ++k) {
                 t.clear();
-                set_run(groups[gi], k, 0.f, 0.f, 0.f, true, false);
-                build_table(groups[gi], slot_class[gi], st->classes, t);
+                run_table(groups[gi], slot_class[gi], st->classes, k, true, t);
                 st->tables.back().grouped_items[k] = static_cast<int32_t>(t.size());
                 tables.push_back(std::move(t));
             }
@@ -1062,6 +1070,34 @@ int run_host_step(malt_state* st, const malt_param_t* params, int32_t n, const m
     return MALT_OK;
 }
 
+// Entries of a launch group's table, `width` (8 or 11) int32 each, from position `total` of out on;
+// returns the new position (counted past the capacity too).
+int64_t write_table(const NsParams& G, int group, int nmat, const std::vector<NsEntry>& table, size_t items,
+                    int32_t* out, int32_t width, int64_t capacity, int64_t total) {
+    for (size_t i = 0; i < items; ++i, ++total) {
+        if (total >= capacity) continue;
+        const NsEntry& e = table[i];
+        const int st = entry_stage(e);
+        const NsClass& C = G.cls[entry_cls(e)];
+        const int kind = ns_op(G, C, st).kind;
+        int32_t* o = out + total * width;
+        o[0] = group;
+        o[1] = st;
+        o[2] = kind;
+        o[3] = e.g;
+        o[4] = e.local;
+        o[5] = e.target > 0 ? (st - 1) * nmat + e.g : -1;
+        o[6] = static_cast<int32_t>(e.target);
+        o[7] = stage_items(kind, C);
+        if (width > 8) {
+            o[8] = C.tile_n;
+            o[9] = entry_cls(e);
+            o[10] = entry_b(e);
+        }
+    }
+    return total;
+}
+
 // malt_ns_plan and malt_muon_ns_plan.
 int ns_plan_of_step(int64_t rows, int64_t cols, int32_t n, const malt_hparams_t* hp, bool raw, malt_ns_op_t* out,
                     int32_t capacity, int32_t* count) {
@@ -1357,22 +1393,38 @@ int malt_ns_schedule(const malt_param_t* params, int32_t n, int32_t ns_steps, in
         NsParams& G = groups[gi];
         set_run(G, ns_steps, 0.f, 0.f, 0.f, false, false);
         build_table(G, slot_class[gi], classes, table);
-        for (const NsEntry& e : table) {
-            if (total < capacity) {
-                const int st = entry_stage(e);
-                const int kind = st % 3;
-                int32_t* o = out + total * 8;
-                o[0] = static_cast<int32_t>(gi);
-                o[1] = st;
-                o[2] = kind;
-                o[3] = e.g;
-                o[4] = e.local;
-                o[5] = e.target > 0 ? (st - 1) * n + e.g : -1;
-                o[6] = static_cast<int32_t>(e.target);
-                o[7] = stage_items(kind, G.cls[entry_cls(e)]);
-            }
-            ++total;
-        }
+        total = write_table(G, static_cast<int>(gi), n, table, table.size(), out, 8, capacity, total);
+    }
+    *count = total;
+    return MALT_OK;
+}
+
+int malt_ns_tables(const malt_param_t* params, int32_t n, const malt_hparams_t* hp, int32_t muon, int32_t* out,
+                   int64_t capacity, int64_t* count) {
+    if (count == nullptr || n < 0 || (n > 0 && params == nullptr) || capacity < 0 || (capacity > 0 && out == nullptr))
+        return MALT_ERR_INVALID_ARG;
+    const int rc = validate_hparams(hp);
+    if (rc != MALT_OK) return rc;
+    for (int i = 0; i < n; ++i)
+        if (params[i].rows <= 0 || params[i].cols <= 0 ||
+            round8(params[i].rows) * round8(params[i].cols) >= (int64_t{1} << 31))
+            return MALT_ERR_UNSUPPORTED;
+    const int k = hp->ns_steps;
+    const bool grouped_run = ns_grouped_run(k, hp->ns_a, hp->ns_b, hp->ns_c, muon != 0);
+    std::vector<MatDesc> hmats;
+    std::vector<ShapeClass> classes;
+    build_classes(params, n, true, hmats, classes);
+    std::vector<NsParams> groups;
+    std::vector<std::vector<int>> slot_class;
+    plan_ns_groups(classes, n, groups, &slot_class);
+    int64_t total = 0;
+    std::vector<NsEntry> table;
+    for (size_t gi = 0; gi < groups.size(); ++gi) {
+        NsParams& G = groups[gi];
+        const bool grouped = grouped_run && any_grouped(G);
+        run_table(G, slot_class[gi], classes, k, grouped, table);
+        const size_t items = grouped ? table.size() : static_cast<size_t>(k) * table_per_iter(G);
+        total = write_table(G, static_cast<int>(gi), n, table, items, out, 11, capacity, total);
     }
     *count = total;
     return MALT_OK;

@@ -39,7 +39,8 @@ EXPORTS = ("malt_init_state", "malt_step", "malter_step", "malt_get_scalars",
            "malt_ns_schedule", "malt_debug_timeout_site", "malt_debug_precond",
            "malt_set_weight_copies", "malt_adamw_init_state", "malt_adamw_step",
            "malt_adamw_get_step", "malt_adamw_set_step", "malt_adamw_destroy_state",
-           "malt_debug_check_guards", "malt_ns_plan", "malt_muon_ns_plan")
+           "malt_debug_check_guards", "malt_ns_plan", "malt_muon_ns_plan",
+           "malt_ns_tables")
 NOALLOC_SCRATCH_FLOATS = 1048576
 KIND_NAMES = ("bind", "stats", "finalize", "prescale", "norms", "ns_gram", "ns_poly", "ns_bx",
               "scalars", "apply", "ns_persistent", "pad")
@@ -155,6 +156,8 @@ def load(build_if_missing: bool = False) -> ctypes.CDLL:
     lib.malt_adamw_destroy_state.argtypes = [vp]
     lib.malt_adamw_destroy_state.restype = None
     lib.malt_ns_schedule.restype = ctypes.c_int
+    lib.malt_ns_tables.argtypes = [P(malt_param_t), i32, P(malt_hparams_t), i32, P(i32), i64, P(i64)]
+    lib.malt_ns_tables.restype = ctypes.c_int
     for name in ("malt_ns_plan", "malt_muon_ns_plan"):
         getattr(lib, name).argtypes = [i64, i64, i32, P(malt_hparams_t), P(malt_ns_op_t), i32, P(i32)]
         getattr(lib, name).restype = ctypes.c_int
@@ -455,25 +458,40 @@ def malt_set_ns_schedule(st, schedule: int):
     _check(load().malt_set_ns_schedule(st, int(schedule)), "malt_set_ns_schedule")
 
 
+def _shape_params(shapes):
+    arr = (malt_param_t * max(len(shapes), 1))()
+    for i, (rows, cols) in enumerate(shapes):
+        arr[i] = malt_param_t(None, MALT_F32, None, MALT_F32, None, None, None, rows, cols)
+    return arr
+
+
+def _table(call, width, where):
+    """call(out or None, capacity, count): the items of a host-side table."""
+    import numpy as np
+    count = ctypes.c_int64(0)
+    _check(call(None, 0, ctypes.byref(count)), where)
+    out = np.zeros((count.value, width), dtype=np.int32)
+    _check(call(out.ctypes.data_as(ctypes.POINTER(ctypes.c_int32)), count.value, ctypes.byref(count)), where)
+    return out
+
+
 def malt_ns_schedule(shapes, ns_steps: int):
     """The work table of the persistent schedule for these (rows, cols)
     shapes, computed on the host by the library (no GPU): an int32 array of
     shape (items, 8) with columns launch group, stage, product kind
     (STAGE_KIND_NAMES), matrix, tile, counter index, counter target, tiles of
     (stage, matrix)."""
-    import numpy as np
-    arr = (malt_param_t * max(len(shapes), 1))()
-    for i, (rows, cols) in enumerate(shapes):
-        arr[i] = malt_param_t(None, MALT_F32, None, MALT_F32, None, None, None, rows, cols)
-    lib = load()
-    count = ctypes.c_int64(0)
-    _check(lib.malt_ns_schedule(arr, len(shapes), ns_steps, None, 0, ctypes.byref(count)),
-           "malt_ns_schedule")
-    out = np.zeros((count.value, 8), dtype=np.int32)
-    _check(lib.malt_ns_schedule(arr, len(shapes), ns_steps,
-                                out.ctypes.data_as(ctypes.POINTER(ctypes.c_int32)),
-                                count.value, ctypes.byref(count)), "malt_ns_schedule")
-    return out
+    arr, lib = _shape_params(shapes), load()
+    return _table(lambda *a: lib.malt_ns_schedule(arr, len(shapes), ns_steps, *a), 8, "malt_ns_schedule")
+
+
+def malt_ns_tables(shapes, hp: malt_hparams_t, muon: bool = False):
+    """The work tables that the persistent launches of a step (a Muon step) of these
+    shapes claim from (no GPU): the columns of malt_ns_schedule, then tile width,
+    class slot and batch slot."""
+    arr, lib = _shape_params(shapes), load()
+    return _table(lambda *a: lib.malt_ns_tables(arr, len(shapes), ctypes.byref(hp), int(muon), *a), 11,
+                  "malt_ns_tables")
 
 
 def malt_ns_plan(rows: int, cols: int, n: int, hp: malt_hparams_t, muon: bool = False):
