@@ -1,6 +1,11 @@
-"""The grouped Newton-Schulz form on frames whose rows and columns differ by many
-decades: every row and column of the direction keeps the accuracy that the
-iterated bf16 form has on it (a CPU model of that form's arithmetic)."""
+"""The grouped Newton-Schulz form (3 to 8 iterations of wide frames).
+
+On frames whose rows and columns differ by many decades every row and column of
+the direction keeps the accuracy that the iterated bf16 form has on it (a CPU
+model of that form's arithmetic).  Each number of iterations, with its own list of
+products and work table, matches the oracle, and one state takes them in turn."""
+import dataclasses
+
 import numpy as np
 import pytest
 
@@ -8,6 +13,7 @@ import paper_2608_05088_gb300.malt as malt
 from paper_2608_05088_gb300 import inputs
 from tests.bf16_ns_model import newton_schulz_bf16
 from tests.gpu_harness import Run
+from tests.test_gpu_schedule import run_both
 from tests.test_ns_plan import graded_frames, is_grouped
 
 pytestmark = pytest.mark.gpu
@@ -56,3 +62,36 @@ def check_slices(run, names, k):
             # bars of tests/test_ns_plan.py
             assert np.sqrt(np.mean(e_new ** 2)) < 1.1 * np.sqrt(np.mean(e_old ** 2)), (name, axis)
             assert e_new.max() < 2.0 * e_old.max(), (name, axis, e_new.max(), e_old.max())
+
+
+# grouped (wide and tall, ragged) and iterated frames in one launch; the second set
+# in 128-wide tiles
+WIDE = ((776, 1560),) * 5 + ((1560, 776),) * 4 + ((520, 520),)
+NARROW = ((256, 4096), (2184, 264), (136, 264))
+
+
+@pytest.mark.parametrize("shapes", [WIDE, NARROW])
+@pytest.mark.parametrize("k", [3, 4, 6, 7, 8])
+def test_each_number_of_iterations_bitwise(shapes, k):
+    wl = inputs.Workload("grouped_k", 82, shapes, "f32", 1.5, 0.02, "malter", 1, ns_steps=k)
+    run_both(wl, 1, schedules=[malt.MALT_NS_PHASED, malt.MALT_NS_PERSISTENT])
+
+
+@pytest.mark.parametrize("variant", ["malter", "muon"])
+@pytest.mark.parametrize("schedule", [malt.MALT_NS_PERSISTENT, malt.MALT_NS_PHASED])
+@pytest.mark.parametrize("shapes,check", [(WIDE, (0, 8, 9)), (NARROW, (0, 1, 2))])
+def test_iterations_change_between_steps(shapes, check, schedule, variant):
+    """One state stepped with every grouped number of iterations and two iterated ones
+    in turn; every step matches the oracle run with the same sequence."""
+    wl = inputs.Workload("grouped_switch", 83, shapes, "f32", 1.0, 0.02, variant, 8)
+    run = Run(wl, check=check)
+    run.opt.set_ns_schedule(schedule)
+    base = run.hp_ref
+    for s, k in enumerate((5, 3, 8, 2, 7, 4, 9, 6)):
+        run.hp_ref = dataclasses.replace(base, ns_steps=k)
+        run.hp = malt.hparams(lr=wl.lr, ns_steps=k)
+        run.step()
+        assert run.status() == malt.MALT_OK, run.opt.timeout_site()
+        for i in check:
+            run.assert_close(i, f"step {s} k={k}")
+    run.close()
