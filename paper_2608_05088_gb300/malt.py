@@ -375,9 +375,10 @@ def adamw_hparams(lr=1e-3, betas=(0.9, 0.95), eps=1e-8) -> malt_adamw_hparams_t:
 
 
 def _float_words(values):
-    """The 32 bits of each value as a float, as ints."""
+    """The 32 bits of each value as a float, as ints (native packing rounds values past
+    the largest float to infinity, as a C cast does; standard packing refuses them)."""
     n = len(values)
-    return struct.unpack(f"<{n}I", struct.pack(f"<{n}f", *values))
+    return struct.unpack(f"{n}I", struct.pack(f"{n}f", *map(float, values)))
 
 
 def adamw_params_array(params):
