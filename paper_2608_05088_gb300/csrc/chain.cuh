@@ -51,7 +51,9 @@ cudaError_t launch_chained(void (*kernel)(Params...), unsigned blocks, unsigned 
     attr[0].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = attr;
     cfg.numAttrs = 1;
-    return cudaLaunchKernelEx(&cfg, kernel, std::forward<Args>(args)...);
+    const cudaError_t e = cudaLaunchKernelEx(&cfg, kernel, std::forward<Args>(args)...);
+    if (e != cudaSuccess) cudaGetLastError();   // reported here, not by a later launch's check
+    return e;
 }
 
 }  // namespace malt

@@ -1068,7 +1068,6 @@ cudaError_t launch_ns_gemm(const NsParams& P, int mode, int grid_pairs, cudaStre
                      mode, 2 * grid_pairs, ns_threads(mode), kSmemBytes, sizeof(NsParams),
                      cudaGetErrorString(e), fa.numRegs, fa.sharedSizeBytes,
                      fa.maxThreadsPerBlock, fa.maxDynamicSharedSizeBytes);
-        cudaGetLastError();
     }
     return e;
 }

@@ -7,6 +7,8 @@ import pytest
 
 import oracle.adamw_ref as aref
 import paper_2608_05088_gb300.malt as malt
+from paper_2608_05088_gb300 import inputs
+from tests.gpu_harness import Run
 from tests.test_gpu_whole_optimizer import AdamRun
 
 pytestmark = pytest.mark.gpu
@@ -62,3 +64,29 @@ def test_noalloc_calls_back_to_back():
     g.manual_seed(76)
     for a, b in zip(plain, calls(False)):
         assert all(torch.equal(x, y) for x, y in zip(a, b))
+
+
+def test_refused_launch_is_reported_once():
+    """A launch that the runtime refuses (into a stream capture that a synchronize has
+    invalidated) fails its own call and no later one."""
+    import torch
+    run = Run(inputs.Workload("refused", 77, ((128, 256),), "f32", 1.0, 0.02, "malt", 1))
+    z = [torch.zeros(s, device="cuda") for s in ((128, 256), (128, 256), (128,), (256,), (128,), (256,))]
+    side = torch.cuda.Stream()
+    assert malt.malt_stats_noalloc(*z, stream=side) == malt.MALT_OK
+    torch.cuda.synchronize()
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.stream(side):
+        graph.capture_begin()
+        with pytest.raises(RuntimeError):
+            side.synchronize()
+        rc = malt.malt_stats_noalloc(*z, stream=side)
+        with pytest.raises(RuntimeError):
+            graph.capture_end()
+    torch.cuda.synchronize()
+    assert rc == malt.MALT_ERR_CUDA
+    assert run.opt.guard_bytes_corrupted() == 0      # checks the last error after its launch
+    run.step()
+    assert run.status() == malt.MALT_OK
+    run.assert_close(0)
+    run.close()
