@@ -604,7 +604,9 @@ __device__ __forceinline__ void apply8(const MatDesc& d, const UserPtrs& up, boo
 __device__ __forceinline__ void apply_block(const MatDesc& d, const UserPtrs& up, int local,
                                             float s, float decay, int tid) {
     constexpr int P = kLdPlain;
-    constexpr int PO = kLdRO;                     // O: written by an earlier launch
+    // O: through L2 only.  The launch that writes it may still run when this one
+    // starts (chain_wait), so it is not read-only for the kernel's lifetime.
+    constexpr int PO = kLdL2;
     const int m = d.m, n = d.n;
     const bool wbf = d.w_bf16 != 0;
     const int32_t total = m * n;
