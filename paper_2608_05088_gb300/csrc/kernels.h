@@ -74,13 +74,12 @@ cudaError_t launch_guards(void* base, const uint64_t* offsets, int32_t n, bool c
                           unsigned long long* bad, cudaStream_t s);
 
 // Newton-Schulz products over up to kMaxClasses shape classes on grid_pairs
-// CTA pairs (clusters of two).  mode kNsPhased: the items
-// [P.item_begin, P.item_end) of one product, static round-robin.
+// CTA pairs (clusters of two).  mode kNsPhased: the P.item_end items of one
+// stage (P.stage), static round-robin.
 // kNsPersistent: the work table P.table, claimed dynamically, each item
 // waiting for its matrix's previous product (P.queue and P.done zeroed by the
 // norms launch).
 cudaError_t launch_ns_gemm(const NsParams& P, int mode, int grid_pairs, cudaStream_t s);
-size_t ns_gemm_smem_bytes();
 int ns_gemm_max_pairs();
 // Opt the GEMM kernel into its shared memory and count the resident CTA pairs,
 // once per device (on the current device; later calls only look it up).

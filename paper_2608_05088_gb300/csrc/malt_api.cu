@@ -328,7 +328,9 @@ int64_t wide_sym_tiles(int64_t p) {
 // one 1280 x 1280 181 / 151, 16 of 256 x 2048 (16 symmetric and 128 B*X tiles)
 // 162 / 134, 8 of 768 x 768 (48 and 72) 162 / 141, one 2048 x 2048 (36 and 64)
 // 246 / 251, 8 of 1024 x 1024 (80 and 128) 193 / 225.  The wide tile loads a quarter
-// less per flop.  narrow_tiles false: 256 always (malt_ns_schedule's tables).
+// less per flop, which tells where reductions are long: the rule counts tiles only,
+// and frames like the 2048 x 2048 lose 2 % by it.  narrow_tiles false: 256 always
+// (malt_ns_schedule's tables).
 constexpr int kNarrowMaxSym = 48, kNarrowMaxBx = 128;
 void build_classes(const malt_param_t* params, int n, bool narrow_tiles, std::vector<MatDesc>& hmats,
                    std::vector<ShapeClass>& classes) {
@@ -830,7 +832,7 @@ SchedCounters sched_counters(const malt_state* st, const malt_hparams_t* hp) {
 // The k Newton-Schulz iterations over every class (after the norms kernel
 // has set 1 / (||Mt|| + ns_eps)).  raw: the frames are not preconditioned (Muon).
 int run_newton_schulz(malt_state* st, const malt_hparams_t* hp, bool raw, cudaStream_t s) {
-    thread_local NsParams P;  // ~17 KB of tensor maps: keep off the stack
+    thread_local NsParams P;  // 22 KB, most of it tensor maps: keep off the stack
     const int k = hp->ns_steps;
     const int max_pairs = ns_gemm_max_pairs();
     const bool grouped_run = ns_grouped_run(k, hp->ns_a, hp->ns_b, hp->ns_c, raw);

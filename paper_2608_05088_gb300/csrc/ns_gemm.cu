@@ -19,8 +19,8 @@
 // grouped form's further p x p products (H A, H A H, the running product of the
 // H) are kPoly operations on other buffers, in fp16; they commute with A, so
 // they are symmetric too and take the same path.  GPT-2 Large (36 layers, k = 5):
-// 17 products in 8.76 ms in place of 15 in 10.4 ms; one 16384 x 4096 matrix at
-// k = 8 2.89 in place of 4.27 ms (both before symmetric tiles were stored once).  The
+// 17 products in 8.24 ms where the iterated form's 15 take 10.12; one 16384 x 4096
+// matrix at k = 8 2.81 where it takes 4.12 ms.  The
 // 1/(||Mt||_F + ns_eps) normalisation is folded into the first iteration's
 // epilogues (A scaled by k^2, X' by k).  The last product's epilogue writes O
 // in W's orientation and per-warp partial sums of O^2 and of D^2 with
@@ -127,8 +127,9 @@ constexpr uint16_t kPairMask = 0x3;
 // Persistent schedule: slots of the item ring, and the readers of each slot: both
 // producers, the even CTA's MMA thread, every epilogue warp and the signal warp of
 // both CTAs.  A slot is free again once its tile has been reported, so a pair holds
-// at most this many claimed tiles: one in the epilogue, one in the MMAs, one in the
-// loads.  More are claimed by pairs that cannot start them yet while others idle:
+// at most this many published tiles (one in the epilogue, one in the MMAs, one in the
+// loads) and one more that its scheduler has claimed and cannot publish yet.  With more
+// slots pairs claim tiles that they cannot start yet while others idle:
 // GPT-2 Small's step takes 1120 us with 3, 1132 with 4 and 1170 with 6, but 1151
 // with 2; GPT-2 Medium and larger sets differ by less than 0.3 % between 3 and 6.
 constexpr int kItemSlots = 3;
@@ -973,8 +974,6 @@ ns_gemm_kernel(const __grid_constant__ NsParams P) {
         tmem_dealloc_pair(tmem_base, kTmemCols);
     }
 }
-
-size_t ns_gemm_smem_bytes() { return kSmemBytes; }
 
 namespace {
 

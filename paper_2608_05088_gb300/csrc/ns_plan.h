@@ -127,7 +127,8 @@ inline bool ns_grouped_run(int k, double a, double b, double c, bool raw, NsScal
 // long enough or the set is large.  Measured at k = 5, us of Newton-Schulz per
 // step, iterated / grouped: one 512 x 1024 108 / 114, 32 of them 204 / 206, one
 // 512 x 2048 127 / 128, one 256 x 4096 155 / 133, 16 of 1024 x 2048 439 / 400,
-// one 2048 x 4096 383 / 339, 8 of 1280 x 5120 727 / 570.
+// one 2048 x 4096 383 / 339, 8 of 1280 x 5120 727 / 570 (at the line itself, as
+// with the 512 x 2048, it is a percent either way).
 // tiles: 256 x 256 tiles of one symmetric product over the set.
 inline bool ns_grouped_shape(int64_t p, int64_t q, int64_t tiles) {
     return q >= 2 * p && 50 * (q - 2 * p) + tiles * p >= 50000;
