@@ -39,7 +39,7 @@ NCU_SUMMARY = os.path.join(ROOT, "profiles", "ns_gemm_gpt2_large_ncu.json")
 # The sources the Newton-Schulz kernel compiles from: the traffic figure of
 # the committed ncu summary holds only while all of them are unchanged.
 NS_SOURCES = [os.path.join(ROOT, "paper_2608_05088_gb300", "csrc", f)
-              for f in ("ns_gemm.cu", "common.cuh", "ptx.cuh")]
+              for f in ("ns_gemm.cu", "common.cuh", "ptx.cuh", "ns_plan.h", "chain.cuh")]
 
 
 def ns_sources_sha256() -> str:
@@ -248,9 +248,9 @@ def peaks():
 
 
 def ncu_tensor_pipe():
-    """Tensor-pipe busy % of peak of the Gram, Poly and B*X launches from the
-    committed ncu summary, weighted by their captured durations (the NS mix
-    of one iteration), or None when a kernel source changed since."""
+    """Tensor-pipe busy % of peak of the Gram, p x p and B*X launches of a step from
+    the committed ncu summary, weighted by their captured durations, or None when
+    a kernel source changed since."""
     try:
         with open(NCU_SUMMARY) as f:
             s = json.load(f)
